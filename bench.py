@@ -533,12 +533,12 @@ def _cdiv(a, b):
 
 def _amp_kernel_kind(tune_result):
     """Which amplitude kernel the tensor-core path of a process runs: the
-    tuner's choice (0 per-lane interpreter, 1 helicity-shared, 2 split), else
-    the untuned default, the per-lane interpreter."""
-    return int(tune_result.get("helicity_shared", 0)) if tune_result else 0
+    tuner's choice (0 per-lane interpreter, 1 helicity-shared, 2 split, 3
+    phased), else the untuned default, the phased kernel."""
+    return int(tune_result.get("helicity_shared", 0)) if tune_result else 3
 
 
-AMP_KERNEL_NAMES = {0: "per-lane", 1: "helicity-shared", 2: "split"}
+AMP_KERNEL_NAMES = {0: "per-lane", 1: "helicity-shared", 2: "split", 3: "phased"}
 
 
 def _jamp_executed_flops(info):
@@ -667,16 +667,17 @@ def run_serve(args):
     if dom_stage == "amplitudes":
         tc = tune.get(dom_nm) or {}
         kind = _amp_kernel_kind(tc)
-        # algorithmic FLOPs of the kernel that ran: the helicity-shared and the
-        # split kernels evaluate (some) wavefunctions once per helicity pattern
-        # of their legs
-        per_event = {1: info["hs_flops_per_event"], 2: info["hsp_flops_per_event"]}.get(
+        # algorithmic FLOPs of the kernel that ran: the phased, the
+        # helicity-shared and the split kernels evaluate (some) wavefunctions
+        # once per helicity pattern of their legs
+        per_event = {1: info["hs_flops_per_event"], 2: info["hsp_flops_per_event"], 3: info["hs_flops_per_event"]}.get(
             kind, H * fl_stage["amplitudes"])
         flop = events_per_launch * per_event
         achieved = flop / (ms_per_launch * 1e-3) / 1e12
         tpe = None if tc.get("forwarding") else TRAFFIC_BYTES_PER_EVENT.get(
             (dom_nm, dom_stage, kind, tc.get("threads"), tc.get("events_per_cta"), tc.get("grid")))
-        kname = {1: "amp_hs_kernel<float> (helicity-shared)", 2: "amp_hsp_kernel<float> (split)"}.get(
+        kname = {1: "amp_hs_kernel<float> (helicity-shared)", 2: "amp_hsp_kernel<float> (split)",
+                 3: "amp_phased_kernel (phased)"}.get(
             kind, "amp_kernel<float> amplitude output" + (" with forwarding" if tc.get("forwarding") else ""))
         roofline = {"bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
                     "frac": achieved / fp32_peak, "traffic": None if tpe is None else tpe * events_per_launch,

@@ -110,21 +110,23 @@ typedef struct {
                             the rounding order for reproducible results); other
                             values -> MEA_E_ARG */
   int helicity_sharing;  /* amplitude stage of the tensor-core path (MEA_PREC_MIXED,
-                            helicity sums): 0 (default) the autotuner chooses
-                            (untuned: the per-lane interpreter) among the per-lane
-                            interpreter (one
-                            lane per event and helicity combination), the
-                            helicity-shared kernel (one warp per event; every
+                            helicity sums): 0 (default) the phased kernel (a CTA per
+                            event, every stored off-shell current once per helicity
+                            pattern of its own legs in shared memory, the
+                            autotuner choosing its CTA size) for MEA_HEL_SUM_NONZERO
+                            of processes with 6 or 7 partons, else the autotuner's
+                            choice (untuned: the per-lane interpreter) among the
+                            kernels below; all apply the same operations to the
+                            same inputs (bit-identical results); 1 per-lane
+                            interpreter (one lane per event and helicity
+                            combination) only, tuned with and without forwarding
+                            each op's output to the next op in registers; 2
+                            helicity-shared kernel only (one warp per event; every
                             off-shell current evaluated once per helicity pattern
-                            of its own legs instead of once per combination) and
-                            the split kernel (the currents of up to n_ext - 3
+                            of its own legs instead of once per combination); 3
+                            split kernel only (the currents of up to n_ext - 3
                             legs shared that way in a prologue, the rest per
-                            lane); all three apply the same operations to the
-                            same inputs (bit-identical results); the per-lane
-                            interpreter is tuned with and without forwarding each
-                            op's output to the next op in registers; 1 per-lane
-                            interpreter only; 2 helicity-shared kernel only; 3
-                            split kernel only; 4 per-lane interpreter with
+                            lane); 4 per-lane interpreter with
                             forwarding only; other values -> MEA_E_ARG */
 } mea_options;
 
@@ -295,7 +297,8 @@ typedef struct {
                             body with one vertex call per diagram was faster */
   int helicity_shared;   /* 1: the helicity-shared amplitude kernel was chosen
                             (threads = 32 x events_per_cta, one warp per event);
-                            2: the split kernel */
+                            2: the split kernel; 3: the phased kernel (threads / 32
+                            warps per event) */
   int forwarding;        /* 1: the per-lane interpreter with each op's output
                             forwarded to the next op in registers (and not stored
                             when nothing else reads it) was chosen */

@@ -575,6 +575,10 @@ static int interp_resident(bool fp64, bool jsm, bool ssm, bool aout, int threads
 AmpConfig plan_amp(const DevProgram& p, bool fp64, int H, int64_t n_events, int num_sms,
                    size_t max_smem, size_t smem_per_sm, int hint) {
   if (p.gen && hint == 0) return plan_generated(p, fp64, H, n_events, num_sms);
+  if (hint == 0 && phased_supported(p, fp64, H)) {
+    const std::vector<AmpConfig> cs = phased_candidates(p, H, n_events, num_sms, max_smem, smem_per_sm);
+    if (!cs.empty()) return *phased_default(cs);
+  }
   if (hint == 0 && p.hsp_only && hsp_supported(p, fp64, H)) {
     // split evaluation only: the candidate with the most resident lanes
     std::vector<AmpConfig> cs = hsp_candidates(p, H, num_sms, max_smem, smem_per_sm);
@@ -698,6 +702,7 @@ std::vector<AmpConfig> candidate_configs(const DevProgram& p, bool fp64, int H, 
     }
     return out;
   }
+  if (phased_supported(p, fp64, H)) return phased_candidates(p, H, n_events, num_sms, max_smem, smem_per_sm);
   if (hs_supported(p, fp64, H)) {
     for (AmpConfig c : hs_candidates(p, H, num_sms, max_smem, smem_per_sm)) out.push_back(cap(c));
     if (p.hs_only) return out;
@@ -767,7 +772,7 @@ size_t jamp_scratch_bytes_needed(const DevProgram& p, bool fp64, const AmpConfig
 size_t slot_scratch_bytes_needed(const DevProgram& p, bool fp64, const AmpConfig& c) {
   if (c.helshare) return hs_arena_bytes(p, c);
   if (c.hsplit) return hsp_area_bytes(p, c);
-  if (c.slots_in_smem) return 0;
+  if (c.slots_in_smem || c.phased) return 0;
   return (size_t)c.grid * p.n_slots * 8 * c.threads * (fp64 ? sizeof(double) : sizeof(float));
 }
 
@@ -800,6 +805,12 @@ cudaError_t launch_amp(const DevProgram& p, bool fp64, const AmpConfig& c, const
                        cudaStream_t s) {
   if (c.grid <= 0) return cudaSuccess;
   cudaError_t err = cudaSuccess;
+  if (c.phased) {
+    if (fp64) return cudaErrorInvalidValue;
+    err = launch_amp_phased(p, c, a, s);
+    if (err == cudaSuccess) ++launch_counter();
+    return err;
+  }
   if (c.helshare || c.hsplit) {
     if (fp64) return cudaErrorInvalidValue;
     err = c.helshare ? launch_amp_hs(p, c, a, s) : launch_amp_hsp(p, c, a, s);

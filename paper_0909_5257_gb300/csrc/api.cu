@@ -23,6 +23,7 @@
 #include "jamp_gemm.h"
 #include "generator.h"
 #include "kernels.h"
+#include "phased.h"
 #include "process.h"
 
 namespace {
@@ -158,10 +159,31 @@ int64_t tc_chunk_events(const mea_process_s* P, int H, int64_t n) {
   return std::max<int64_t>(1, std::min<int64_t>(n, (int64_t)(bytes / std::max<size_t>(per_event, 1))));
 }
 
-// Launch configuration of the amplitude-output interpreter for H lanes per event.
-mea::AmpConfig tc_amp_config(const mea_process_s* P, const mea::DevProgram& dp, int H, int64_t cn) {
-  mea::AmpConfig c = mea::cached_plan(const_cast<mea_process_s*>(P), dp, false, true, H, cn);
-  if (P->tuned[0].grid > 0 && P->tuned_H[0] == H) {  // configuration chosen by mea_autotune
+// Warps per CTA of the phased amplitude kernel for a chunk of cn events: the
+// shape that keeps the most warps on an SM, counting only the CTAs that the
+// chunk's events fill; the tuned shape (or, untuned, the plan's) on a tie.
+mea::AmpConfig phased_config(const mea_process_s* P, int64_t cn) {
+  const mea::AmpConfig* best = mea::phased_default(P->ph_cands);
+  if (P->tuned[0].grid > 0 && P->tuned[0].phased) best = &P->tuned[0];
+  const int64_t fill = (cn + P->num_sms - 1) / P->num_sms;  // CTAs per SM with an event
+  auto warps = [&](const mea::AmpConfig& c) { return std::min<int64_t>(c.per_sm, fill) * c.threads; };
+  if (fill < best->per_sm)
+    for (const mea::AmpConfig& c : P->ph_cands)
+      if (warps(c) > warps(*best)) best = &c;
+  mea::AmpConfig c = *best;
+  c.grid = (int)std::min<int64_t>((int64_t)c.per_sm * P->num_sms, std::max<int64_t>(cn, 1));
+  return c;
+}
+
+// Launch configuration of the amplitude-output kernel for H lanes per event
+// (lda: the row stride of the diagram amplitudes; the phased kernel's byte
+// strides are 32-bit).
+mea::AmpConfig tc_amp_config(const mea_process_s* P, const mea::DevProgram& dp, int H, int64_t cn, int64_t lda) {
+  if (mea::phased_supported(dp, false, H) && !P->ph_cands.empty() && lda <= mea::kPhasedMaxLda) return phased_config(P, cn);
+  mea::DevProgram lanes = dp;
+  lanes.ph_units = nullptr;
+  mea::AmpConfig c = mea::cached_plan(const_cast<mea_process_s*>(P), lanes, false, true, H, cn);
+  if (P->tuned[0].grid > 0 && P->tuned_H[0] == H && !P->tuned[0].phased) {  // configuration chosen by mea_autotune
     c = P->tuned[0];
     int64_t tiles = (cn + c.E_cta - 1) / c.E_cta;
     if (tiles < c.grid) c.grid = (int)std::max<int64_t>(tiles, 1);
@@ -221,7 +243,7 @@ mea_status do_evaluate_tc(mea_process_s* P, mea::EvalScratch& S, const double* m
   cg.pairval = reinterpret_cast<double*>(S.pairval.p);
   for (int64_t c0 = 0; c0 < n; c0 += chunk) {
     const int64_t cn = std::min(chunk, n - c0);
-    mea::AmpConfig c = tc_amp_config(P, dp, H, cn);
+    mea::AmpConfig c = tc_amp_config(P, dp, H, cn, lda);
     mea::AmpLaunch a;
     a.mom = mom + (size_t)c0 * n_ext * 4;
     a.n_events = cn;
@@ -559,7 +581,45 @@ mea_status mea_create_process(const int* pdg, int n_ext, const mea_options* opts
       std::vector<__half>().swap(P->jmap.tiles);
     }
   }
-  if (P->jmap.ok && P->opts.helicity_sharing != 2 && P->opts.helicity_sharing != 3) {
+  bool phased = false;
+  if (P->jmap.ok && P->opts.helicity_sharing == 0) {
+    // phased layout for the tensor-core path's amplitude stage; processes it
+    // does not cover (and helicity_sharing 1..4) take the kernels below
+    try {
+      P->ph = mea::build_phased(G, P->jmap.weight, mea::phased_max_area(G, P->smem_optin));
+      phased = true;
+    } catch (std::exception&) {
+    }
+  }
+  if (phased) {
+    const uint32_t* dr = nullptr;
+    const mea::PhUnit* du = nullptr;
+    const mea::PhSet* ds = nullptr;
+    const uint8_t* dv = nullptr;
+    const int* de = nullptr;
+    if ((e = upload(P, P->ph.rec, &dr)) != cudaSuccess || (e = upload(P, P->ph.units, &du)) != cudaSuccess ||
+        (e = upload(P, P->ph.sets, &ds)) != cudaSuccess || (e = upload(P, P->ph.hv, &dv)) != cudaSuccess ||
+        (e = upload(P, P->ph.phase_end, &de)) != cudaSuccess) {
+      destroy(P);
+      return fail(MEA_E_CUDA, std::string("mea_create_process: ") + cudaGetErrorString(e));
+    }
+    D.ph_rec = dr;
+    D.ph_units = du;
+    D.ph_sets = ds;
+    D.ph_hv = dv;
+    D.ph_end = de;
+    D.ph_phases = (int)P->ph.phase_end.size();
+    D.ph_area = P->ph.area;
+    D.ph_H = P->ph.H;
+    P->ph = mea::PhProgram();
+    mea::DevProgram dp = D;
+    dp.gen = nullptr;
+    dp.n_colour = 0;
+    P->ph_cands = mea::phased_candidates(dp, D.ph_H, (int64_t)1 << 40, P->num_sms, P->smem_optin, P->smem_per_sm);
+    phased = !P->ph_cands.empty();
+    if (!phased) D.ph_units = nullptr;
+  }
+  if (P->jmap.ok && !phased && P->opts.helicity_sharing != 2 && P->opts.helicity_sharing != 3) {
     D.fwd_only = P->opts.helicity_sharing == 4;
     // register forwarding for the amplitude-output interpreter (helshare.h)
     const std::vector<uint8_t> fw = mea::build_forwarding_flags(G);
@@ -570,7 +630,7 @@ mea_status mea_create_process(const int* pdg, int n_ext, const mea_options* opts
     }
     D.fwd = dfw;
   }
-  if (P->hsp_ok && P->jmap.ok && (P->opts.helicity_sharing == 0 || P->opts.helicity_sharing == 3)) {
+  if (P->hsp_ok && P->jmap.ok && !phased && (P->opts.helicity_sharing == 0 || P->opts.helicity_sharing == 3)) {
     // split layout for the tensor-core path's amplitude stage
     const uint32_t* dt = nullptr;
     const mea::HsOp *dr = nullptr, *dmr = nullptr;
@@ -590,7 +650,7 @@ mea_status mea_create_process(const int* pdg, int n_ext, const mea_options* opts
     D.hsp_area = P->hsp.area;
     D.hsp_only = P->opts.helicity_sharing == 3;
   }
-  if (P->hs_ok && P->jmap.ok && (P->opts.helicity_sharing == 0 || P->opts.helicity_sharing == 2)) {
+  if (P->hs_ok && P->jmap.ok && !phased && (P->opts.helicity_sharing == 0 || P->opts.helicity_sharing == 2)) {
     // helicity-shared layout for the tensor-core path's amplitude stage
     const mea::HsOp* dhs = nullptr;
     if ((e = upload(P, P->hs.ops, &dhs)) != cudaSuccess) {

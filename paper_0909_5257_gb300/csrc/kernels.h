@@ -13,6 +13,8 @@ struct DevProgram;
 struct AmpConfig;
 struct AmpLaunch;
 struct HsOp;
+struct PhUnit;
+struct PhSet;
 
 // A straight-line per-process kernel emitted by codegen.cpp at build time.
 struct GenEntry {
@@ -63,6 +65,16 @@ struct DevProgram {
   int hsp_n_main = 0;
   int hsp_area = 0;                     // prologue variants per event
   bool hsp_only = false;                // amplitude-output mode: plan and tune the split kernel only
+  // phased evaluation (phased.h), or null: units, their records, the end of
+  // each phase, leg-set tables and the variant of every leg set per combination
+  const PhUnit* ph_units = nullptr;
+  const uint32_t* ph_rec = nullptr;
+  const int* ph_end = nullptr;
+  const PhSet* ph_sets = nullptr;
+  const uint8_t* ph_hv = nullptr;
+  int ph_phases = 0;
+  int ph_area = 0;
+  int ph_H = 0;
   // per op: bits 0..3 input k is the previous op's output, bit 4 the op's
   // output is read only by the next op (amplitude-output interpreter with
   // register forwarding), or null
@@ -106,6 +118,7 @@ struct AmpConfig {
   bool fwd = false;       // amplitude-output interpreter: the previous op's output forwarded in registers
   bool hsplit = false;    // amplitude-output mode: the split kernel (amp_hsp_kernel, amp_hs_kernel.cu):
                           // E_cta events x H lanes; slots_in_smem = its prologue area in shared memory
+  bool phased = false;    // amplitude-output mode: the phased kernel (amp_phased_kernel.cu), a CTA per event
   bool helshare = false;  // amplitude-output mode: the helicity-shared kernel (amp_hs_kernel.cu):
                           // one warp per event, E_cta = warps per CTA, regvar its register
                           // variant (0: 64 registers, 1: uncapped)
@@ -145,6 +158,15 @@ size_t hsp_smem_bytes(const DevProgram& p, int events, bool area_in_smem);
 size_t hsp_area_bytes(const DevProgram& p, const AmpConfig& c);
 std::vector<AmpConfig> hsp_candidates(const DevProgram& p, int H, int num_sms, size_t max_smem, size_t smem_per_sm);
 cudaError_t launch_amp_hsp(const DevProgram& p, const AmpConfig& c, const AmpLaunch& a, cudaStream_t s);
+
+// Phased kernel: every stored wavefunction in shared memory, a CTA per event.
+constexpr int64_t kPhasedMaxLda = 0x3fffffff;
+bool phased_supported(const DevProgram& p, bool fp64, int H);
+int phased_max_area(const Program& P, size_t max_smem);  // variants that fit a CTA's shared memory
+std::vector<AmpConfig> phased_candidates(const DevProgram& p, int H, int64_t n_events, int num_sms, size_t max_smem,
+                                         size_t smem_per_sm);
+const AmpConfig* phased_default(const std::vector<AmpConfig>& cands);  // the untuned shape
+cudaError_t launch_amp_phased(const DevProgram& p, const AmpConfig& c, const AmpLaunch& a, cudaStream_t s);
 
 // Helicity sum + flags for the split colour stage: me2 = 1/4 sum_h pairval.
 // With jabs ([n_splits][n_events*H] sums of |J|), pair_kappa holds sum |c A|

@@ -15,6 +15,7 @@
 #include "helshare.h"
 #include "jamp_gemm.h"
 #include "kernels.h"
+#include "phased.h"
 
 namespace mea {
 
@@ -58,6 +59,8 @@ struct mea_process_s {
   bool hs_ok = false;
   mea::HsSplitProgram hsp;  // split layout of prog (valid when hsp_ok)
   bool hsp_ok = false;
+  mea::PhProgram ph;               // phased layout (until uploaded)
+  std::vector<mea::AmpConfig> ph_cands;  // launch shapes of the phased kernel
   mea::DevProgram dev;
   mea_options opts;
   int device = 0;
