@@ -544,8 +544,12 @@ AMP_KERNEL_NAMES = {0: "per-lane", 1: "helicity-shared", 2: "split", 3: "phased"
 def _jamp_executed_flops(info):
     """Tensor FLOPs the colour-amplitude GEMM executes per (event, helicity)
     pair: Re and Im rows x 2 FLOP x padded diagrams x padded colour columns
-    x 3 digit planes (tiles of 64 diagrams, column splits of at most 128)."""
+    x 3 digit planes (tiles of 64 diagrams, column splits of at most 128).
+    Pure-gluon processes contract (n - 2)! of their (n - 1)!/2 colour
+    amplitudes; chunks without a coefficient of a split are not counted out."""
     m, kd = info["n_colour_amplitudes"], info["n_diagrams"]
+    if info["n_colour"] == 2 * m:
+        m = m * 2 // (info["n_ext"] - 1)
     nc = min(128, _cdiv(m, 16) * 16)
     splits = _cdiv(m, nc)
     nc = min(nc, _cdiv(_cdiv(m, splits), 16) * 16)

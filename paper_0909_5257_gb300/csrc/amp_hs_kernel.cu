@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(CAP == 0 ? 128 : 256, CAP == 0 ? 8 : 1)
           __syncwarp();  // the variants are read by other lanes from here on
         } else {
           const float wd = __ldg(P.amp_w + d_amp);
-          float* col = A.amp_out + (size_t)d_amp * A.lda;
+          float* col = A.amp_out + (size_t)__ldg(P.amp_row + d_amp) * A.lda;
 #pragma unroll
           for (int j = 0; j < NP; ++j) {
             const int h = lane + 32 * j;
@@ -449,7 +449,7 @@ __global__ void __launch_bounds__(512) amp_hsp_kernel(const DevProgram P, const 
           tr = hs_produce(op, P, x, et, mt, g, gg);
         } else {
           const cx<float> amp = hs_amplitude(op, x, mt, g, gg);
-          *reinterpret_cast<float2*>(A.amp_out + (size_t)d_amp * A.lda + 2 * pair) = make_float2(amp.r, amp.i);
+          *reinterpret_cast<float2*>(A.amp_out + (size_t)__ldg(P.amp_row + d_amp) * A.lda + 2 * pair) = make_float2(amp.r, amp.i);
           const float a_r = fabsf(amp.r), a_i = fabsf(amp.i);
           finite = finite && isfinite(a_r) && isfinite(a_i);
           mx_re = fmaxf(mx_re, a_r);

@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(kMaxThreads) amp_kernel(const DevProgram P, co
       // colour amplitudes through its colour entries
       auto take_amp = [&](uint32_t col_begin, uint32_t col_count, const cx<R>& amp) {
         if (AOUT) {
-          float2* dst = reinterpret_cast<float2*>(A.amp_out + (size_t)d_amp * A.lda + 2 * pair);
+          float2* dst = reinterpret_cast<float2*>(A.amp_out + (size_t)__ldg(P.amp_row + d_amp) * A.lda + 2 * pair);
           *dst = make_float2((float)amp.r, (float)amp.i);
           const float ar = fabsf((float)amp.r), ai = fabsf((float)amp.i);
           finite_amps = finite_amps && isfinite(ar) && isfinite(ai);

@@ -218,13 +218,19 @@ mea_status do_evaluate_tc(mea_process_s* P, mea::EvalScratch& S, const double* m
   jg.lda = lda;
   jg.rowmax = reinterpret_cast<const float*>(S.rowmax.p);
   jg.kd = JM.kd;
-  jg.kpad = JM.kpad;
   jg.m = m;
+  jg.mb = JM.mb;
   jg.nc = JM.nc;
   jg.n_splits = JM.n_splits;
   jg.q = JM.q;
   jg.cfac = JM.cfac;
   jg.tiles = P->jmap_tiles;
+  jg.chunks = P->jmap_chunks;
+  jg.split_begin = P->jmap_begin;
+  jg.n_chunks = (int)JM.chunks.size();
+  jg.kk_index = P->jmap_kk_index;
+  jg.kk_term = P->jmap_kk_term;
+  jg.kk_terms = (int)JM.kk_term.size();
   jg.J = reinterpret_cast<float*>(S.jbuf.p);
   jg.ldj = ldj;
   jg.jabs = reinterpret_cast<float*>(S.jabs.p);
@@ -572,12 +578,18 @@ mea_status mea_create_process(const int* pdg, int n_ext, const mea_options* opts
     if (P->jmap.ok) {
       const __half* dt = nullptr;
       const float* dw = nullptr;
-      if ((e = upload(P, P->jmap.tiles, &dt)) != cudaSuccess || (e = upload(P, P->jmap.weight, &dw)) != cudaSuccess) {
+      const int* dr = nullptr;
+      if ((e = upload(P, P->jmap.tiles, &dt)) != cudaSuccess || (e = upload(P, P->jmap.weight, &dw)) != cudaSuccess ||
+          (e = upload(P, P->jmap.row, &dr)) != cudaSuccess || (e = upload(P, P->jmap.chunks, &P->jmap_chunks)) != cudaSuccess ||
+          (e = upload(P, P->jmap.split_begin, &P->jmap_begin)) != cudaSuccess ||
+          (e = upload(P, P->jmap.kk_index, &P->jmap_kk_index)) != cudaSuccess ||
+          (e = upload(P, P->jmap.kk_term, &P->jmap_kk_term)) != cudaSuccess) {
         destroy(P);
         return fail(MEA_E_CUDA, std::string("mea_create_process: ") + cudaGetErrorString(e));
       }
       P->jmap_tiles = dt;
       D.amp_w = dw;
+      D.amp_row = dr;
       std::vector<__half>().swap(P->jmap.tiles);
     }
   }
@@ -586,7 +598,7 @@ mea_status mea_create_process(const int* pdg, int n_ext, const mea_options* opts
     // phased layout for the tensor-core path's amplitude stage; processes it
     // does not cover (and helicity_sharing 1..4) take the kernels below
     try {
-      P->ph = mea::build_phased(G, P->jmap.weight, mea::phased_max_area(G, P->smem_optin));
+      P->ph = mea::build_phased(G, P->jmap.weight, P->jmap.row, mea::phased_max_area(G, P->smem_optin));
       phased = true;
     } catch (std::exception&) {
     }

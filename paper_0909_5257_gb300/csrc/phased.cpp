@@ -50,7 +50,8 @@ void check(bool ok, const char* why) {
 
 }  // namespace
 
-PhProgram build_phased(const Program& P, const std::vector<float>& weight, int max_area) {
+PhProgram build_phased(const Program& P, const std::vector<float>& weight,
+                       const std::vector<int>& row, int max_area) {
   const int n = P.n_ext, H = P.n_hel;
   check(n >= 6 && n <= 7, "6 or 7 legs");
   check(H >= 1 && H <= 128, "at most 128 combinations");
@@ -97,7 +98,8 @@ PhProgram build_phased(const Program& P, const std::vector<float>& weight, int m
       holder.at(op.out) = i;
     }
   }
-  check(n_amp < 0x7FFF && weight.size() == (size_t)n_amp, "diagram ordinals of 15 bits");
+  check(n_amp < 0x7FFF && weight.size() == (size_t)n_amp && row.size() == weight.size(),
+        "diagram ordinals of 15 bits");
 
   // fused: read once, by a contraction, with n - 2 legs and at least two rounds
   std::vector<char> fused(n_ops, 0), stored(n_ops, 0);
@@ -291,7 +293,7 @@ PhProgram build_phased(const Program& P, const std::vector<float>& weight, int m
               for (int k = 0; k < 4; ++k) r.d[k] = kPhNone;
               for (int k = 0; k < np; ++k) {
                 const int a = g.second[s.second[p0 + k]][f];
-                r.d[k] = (uint16_t)(ordinal[a] | ((P.ops[a].leg & 2u) ? 0x8000 : 0));
+                r.d[k] = (uint16_t)(row[ordinal[a]] | ((P.ops[a].leg & 2u) ? 0x8000 : 0));
                 r.w[k] = weight[ordinal[a]];
               }
               put(&r, sizeof r);
@@ -380,7 +382,7 @@ PhProgram build_phased(const Program& P, const std::vector<float>& weight, int m
           if (op.type == OP_JVV) { r.r[0] = (uint8_t)op.min[0]; r.r[1] = (uint8_t)op.min[1]; }
           r.r[2] = (uint8_t)op.mout;
           r.p = (uint16_t)off[p];
-          r.d = (uint16_t)(ordinal[a] | ((P.ops[a].leg & 2u) ? 0x8000 : 0));
+          r.d = (uint16_t)(row[ordinal[a]] | ((P.ops[a].leg & 2u) ? 0x8000 : 0));
           r.w = weight[ordinal[a]];
           put(&r, sizeof r);
         }
@@ -414,14 +416,14 @@ PhProgram build_phased(const Program& P, const std::vector<float>& weight, int m
           PhGenericRec r{};
           r.type = op.type;
           r.flags = (uint8_t)op.leg;
-          r.d = (uint16_t)ordinal[g.second[b + q]];
+          r.d = (uint16_t)row[ordinal[g.second[b + q]]];
           for (int j = 0; j < op.n_in; ++j) {
             const int s = src[4 * (size_t)g.second[b + q] + j];
             r.in[j] = (uint16_t)off[s];
             r.m[j] = (uint8_t)legs[s];
           }
           for (int j = 0; j < 3; ++j) r.r[j] = (uint8_t)op.min[j];
-          r.w = weight[r.d];
+          r.w = weight[ordinal[g.second[b + q]]];
           put(&r, sizeof r);
         }
         c.cost = 60 + 150.0 * (double)k;

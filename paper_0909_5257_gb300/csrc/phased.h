@@ -116,8 +116,9 @@ struct PhProgram {
 };
 
 // weight[d]: sum of the colour coefficients' magnitudes of diagram d
-// (JampMap::weight).  Throws std::runtime_error when the program does not have
+// (JampMap::weight), row[d] its row in the amplitude buffer (JampMap::row).  Throws std::runtime_error when the program does not have
 // the structure above or its area exceeds max_area variants.
-PhProgram build_phased(const Program& P, const std::vector<float>& weight, int max_area);
+PhProgram build_phased(const Program& P, const std::vector<float>& weight,
+                       const std::vector<int>& row, int max_area);
 
 }  // namespace mea

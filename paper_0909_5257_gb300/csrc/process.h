@@ -85,7 +85,9 @@ struct mea_process_s {
   int* status = nullptr;
   // diagram -> colour-amplitude map for the tensor-core colour-amplitude stage
   mea::JampMap jmap;                  // host description (tiles released after upload)
-  const __half* jmap_tiles = nullptr;  // device copy of the coefficient tiles
+  const __half* jmap_tiles = nullptr;  // device copies of its tables
+  const int *jmap_chunks = nullptr, *jmap_begin = nullptr;
+  const uint16_t *jmap_kk_index = nullptr, *jmap_kk_term = nullptr;
   // host-buffer pipeline
   void* pin_in[2] = {nullptr, nullptr};
   void* pin_out[2] = {nullptr, nullptr};

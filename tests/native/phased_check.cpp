@@ -72,7 +72,12 @@ int main(int argc, char** argv) {
     const int n = P.n_ext, H = P.n_hel;
     std::vector<float> weight(P.n_diagrams);
     for (int d = 0; d < P.n_diagrams; ++d) weight[d] = 1.f + (float)(d % 7);
-    const PhProgram Q = build_phased(P, weight, 6800);
+    std::vector<int> row_of(P.n_diagrams), row(P.n_diagrams);  // a permutation
+    for (int d = 0; d < P.n_diagrams; ++d) row[d] = (int)((d * 5LL + 3) % P.n_diagrams);
+    if (P.n_diagrams % 5 == 0)
+      for (int d = 0; d < P.n_diagrams; ++d) row[d] = P.n_diagrams - 1 - d;
+    for (int d = 0; d < P.n_diagrams; ++d) row_of[row[d]] = d;
+    const PhProgram Q = build_phased(P, weight, row, 6800);
 
     std::mt19937_64 rng(0x5eed + a);
     auto u = [&]() { return std::uniform_real_distribution<double>(-1.0, 1.0)(rng); };
@@ -91,7 +96,7 @@ int main(int argc, char** argv) {
           for (int m = 0; m < 4; ++m) q[m] += leg[4 * l + m];
       q[4] = 1.0 / (q[0] * q[0] - q[1] * q[1] - q[2] * q[2] - q[3] * q[3]);
     }
-    auto row = [&](int r) -> const double* {
+    auto mrow = [&](int r) -> const double* {
       if (5 * (size_t)r + 5 > in.mt.size()) { fault("event-table row"); return in.mt.data(); }
       return &in.mt[5 * (size_t)r];
     };
@@ -107,11 +112,11 @@ int main(int argc, char** argv) {
         const int n_in = op.type == OP_EXT ? 0 : op.n_in;
         for (int k = 0; k < n_in; ++k) x[k] = slots[op.in[k]];
         if (is_amp_op(op.type))
-          ref[(size_t)h * P.n_diagrams + d++] = closed(op.type, op.leg, x, row(op.min[0]), row(op.min[1]), row(op.min[2]));
+          ref[(size_t)h * P.n_diagrams + d++] = closed(op.type, op.leg, x, mrow(op.min[0]), mrow(op.min[1]), mrow(op.min[2]));
         else if (op.type == OP_EXT)
           slots[op.out] = in.ext[op.leg][P.hel[(size_t)h * n + op.leg] > 0];
         else
-          slots[op.out] = made(op.type, op.leg, x, row(op.min[0]), row(op.min[1]), row(op.min[2]), row(op.mout));
+          slots[op.out] = made(op.type, op.leg, x, mrow(op.min[0]), mrow(op.min[1]), mrow(op.min[2]), mrow(op.mout));
       }
     }
 
@@ -127,7 +132,8 @@ int main(int argc, char** argv) {
       };
       std::vector<std::pair<int, V>> made_here;
       auto take = [&](cx<double> z, uint32_t d, float w, uint32_t h) {
-        const uint32_t dd = d & 0x7fffu;
+        if ((d & 0x7fffu) >= (uint32_t)P.n_diagrams) { fault("row"); return; }
+        const uint32_t dd = (uint32_t)row_of[d & 0x7fffu];
         if (dd >= (uint32_t)P.n_diagrams || h >= (uint32_t)H) { fault("diagram or combination"); return; }
         if (w != weight[dd]) fault("weight");
         if (d & 0x8000u) z = -z;
@@ -149,7 +155,7 @@ int main(int argc, char** argv) {
               const int n_in = U.op == OP_EXT ? 0 : (U.op == OP_JGGG || U.op == OP_PGGGG ? 3 : 2);
               for (int j = 0; j < n_in; ++j) x[j] = ld(it.in[j]);
               if (U.op == OP_EXT) y = in.ext.at(it.x & 15)[it.x >> 4];
-              else y = made(U.op, it.x, x, row(it.r[0]), row(it.r[1]), row(it.r[2]), row(it.r[2]));
+              else y = made(U.op, it.x, x, mrow(it.r[0]), mrow(it.r[1]), mrow(it.r[2]), mrow(it.r[2]));
               if (it.out >= Q.area) fault("output outside the area");
               else made_here.push_back({it.out, y});
             }
@@ -162,7 +168,7 @@ int main(int argc, char** argv) {
               rec(2 * t, &c, sizeof c);
               V x[4];
               for (int j = 0; j < (U.op == OP_JGGG ? 3 : 2); ++j) x[j] = ld(c.in[j] + T.sub[c.m[j]][lane]);
-              const V y = made(U.op, 0, x, row(c.r[0]), row(c.r[1]), row(c.r[2]), row(c.r[2]));
+              const V y = made(U.op, 0, x, mrow(c.r[0]), mrow(c.r[1]), mrow(c.r[2]), mrow(c.r[2]));
               for (int r = 0; r < kPhRounds; ++r)
                 if (T.uh[r][lane] != kPhNone)
                   take(part_contract<double>(y, ld(c.p + (T.uh[r][lane] & 255)), c.plain != 0, false), c.d, c.w, T.uh[r][lane] >> 8);
@@ -187,7 +193,7 @@ int main(int argc, char** argv) {
                 V x[4];
                 const int n_in = c.type == OP_AGGGG ? 4 : (c.type == OP_ADOT ? 2 : 3);
                 for (int j = 0; j < n_in; ++j) x[j] = ld(c.in[j] + Q.hv[128 * c.m[j] + h]);
-                take(closed(c.type, c.flags, x, row(c.r[0]), row(c.r[1]), row(c.r[2])), c.d, c.w, h);
+                take(closed(c.type, c.flags, x, mrow(c.r[0]), mrow(c.r[1]), mrow(c.r[2])), c.d, c.w, h);
               }
             }
           }
