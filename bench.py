@@ -556,6 +556,12 @@ def _jamp_executed_flops(info):
     return 2 * 2 * (_cdiv(kd, 64) * 64) * (splits * nc) * 3
 
 
+def _lanes_share(info):
+    """Share of the helicity combinations that is evaluated: pure-gluon
+    processes evaluate one of every pair of flipped combinations."""
+    return 0.5 if info["n_colour"] == 2 * info["n_colour_amplitudes"] else 1.0
+
+
 def _colour_sum_executed_flops(info):
     """Tensor FLOPs the colour-sum GEMM executes per pair: 2 rows x 2 FLOP x
     padded K x padded N x MMAs per K step (3 for the 3-way split of J when the
@@ -661,7 +667,7 @@ def run_serve(args):
     dom_nm, dom_stage = max(share, key=share.get)
     tot_share = sum(share.values())
     info = procs[dom_nm].info
-    H = info["n_hel_nonzero"]
+    H = int(info["n_hel_nonzero"] * _lanes_share(info))  # combinations evaluated
     fl_stage = _stage_flops(info, H)
     peaks, peak_src = _peaks()
     bf16_sus = peaks.get("bf16_tflops_sustained", 1700.0)
@@ -676,6 +682,8 @@ def run_serve(args):
         # once per helicity pattern of their legs
         per_event = {1: info["hs_flops_per_event"], 2: info["hsp_flops_per_event"], 3: info["hs_flops_per_event"]}.get(
             kind, H * fl_stage["amplitudes"])
+        if kind in (1, 2, 3):
+            per_event *= _lanes_share(info)
         flop = events_per_launch * per_event
         achieved = flop / (ms_per_launch * 1e-3) / 1e12
         tpe = None if tc.get("forwarding") else TRAFFIC_BYTES_PER_EVENT.get(
@@ -702,7 +710,7 @@ def run_serve(args):
     tensor = {}
     for nm in names:
         inf = procs[nm].info
-        h = inf["n_hel_nonzero"]
+        h = int(inf["n_hel_nonzero"] * _lanes_share(inf))
         f = _stage_flops(inf, h)
         for stg, exec_flop in (("colour_amplitudes", _jamp_executed_flops(inf)),
                                ("colour_sum", _colour_sum_executed_flops(inf))):

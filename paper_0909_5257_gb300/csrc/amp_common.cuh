@@ -225,7 +225,13 @@ __device__ __forceinline__ void tile_prep(const DevProgram& P, const AmpLaunch& 
   }
 }
 
-// Phase 2: thread e < E sums the H helicity lanes of its event in fixed order,
+// Lane of helicity combination h in a sum of paired ? 2 H : H combinations over
+// H lanes (generator.h, HelLanes).
+__device__ __forceinline__ int hel_lane(int h, int H, bool paired) {
+  return paired && h >= H ? 2 * H - 1 - h : h;
+}
+
+// Phase 2: thread e < E sums the helicity combinations of its event in fixed order,
 // applies the 1/4 helicity average, writes me2 and the flags, and appends
 // flagged events to the re-evaluation list.
 template <bool F32>
@@ -239,10 +245,11 @@ __device__ __forceinline__ void tile_finish(const AmpLaunch& A, int t, int E, in
       if (evr < n) {
         int64_t gev = listed ? (int64_t)A.event_list[evr] : evr;
         double s = 0.0, wk = 0.0;
-        for (int hh = 0; hh < H; ++hh) {
-          double v = res[t * H + hh];
+        for (int hh = 0; hh < (A.paired ? 2 * H : H); ++hh) {
+          const int k = t * H + hel_lane(hh, H, A.paired);
+          double v = res[k];
           s += v;
-          wk += v * (double)kap[t * H + hh];
+          wk += v * (double)kap[k];
         }
         double me = 0.25 * s;
         A.me2[gev] = me;

@@ -430,8 +430,8 @@ __global__ void finish_kernel(const AmpLaunch A, int H, const double* pairval, c
   if (e >= A.n_events) return;
   const int64_t n_pairs = A.n_events * H;
   double s = 0.0, wk = 0.0;
-  for (int h = 0; h < H; ++h) {
-    const int64_t p = e * H + h;
+  for (int h = 0; h < (A.paired ? 2 * H : H); ++h) {
+    const int64_t p = e * H + hel_lane(h, H, A.paired);
     double v = pairval[p];
     float k = pk[p];
     if (jabs) {

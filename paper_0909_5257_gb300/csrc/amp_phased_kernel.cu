@@ -373,8 +373,8 @@ bool phased_supported(const DevProgram& p, bool fp64, int H) {
   return !fp64 && p.ph_units != nullptr && p.n_colour == 0 && H == p.ph_H;
 }
 
-int phased_max_area(const Program& P, size_t max_smem) {
-  const size_t rest = ph_smem(0, event_table_stride(P.n_ext, (int)P.masks.size()), P.n_hel);
+int phased_max_area(const Program& P, int H, size_t max_smem) {
+  const size_t rest = ph_smem(0, event_table_stride(P.n_ext, (int)P.masks.size()), H);
   return rest < max_smem ? (int)((max_smem - rest) / 32) : 0;
 }
 

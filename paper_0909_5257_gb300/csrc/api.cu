@@ -196,7 +196,7 @@ mea_status do_evaluate_tc(mea_process_s* P, mea::EvalScratch& S, const double* m
   const mea::Program& G = P->prog;
   const mea::JampMap& JM = P->jmap;
   const int n_ext = G.n_ext;
-  const int H = (hm == MEA_HEL_SUM_NONZERO) ? G.n_hel : (1 << n_ext);
+  const int H = (hm == MEA_HEL_SUM_NONZERO) ? P->lanes.n : (1 << n_ext);
   const int m = G.n_jamp;
   const int ldj = ((m + 15) / 16) * 16;
   const int64_t chunk = tc_chunk_events(P, H, n);
@@ -254,6 +254,7 @@ mea_status do_evaluate_tc(mea_process_s* P, mea::EvalScratch& S, const double* m
     a.mom = mom + (size_t)c0 * n_ext * 4;
     a.n_events = cn;
     a.hel_mode = (int)hm;
+    a.paired = P->lanes.paired && hm == MEA_HEL_SUM_NONZERO;
     a.me2 = me2 + c0;
     a.flags = flags ? flags + c0 : nullptr;
     a.flag_threshold = (float)P->opts.flag_threshold;
@@ -339,7 +340,7 @@ mea_status do_evaluate(mea_process_s* P, mea::EvalScratch& S, const double* mom,
   maybe_autotune(P, mom, n, hm, prec, me2, s);
   if (use_tensor_colour(P, prec, hm)) return do_evaluate_tc(P, S, mom, n, hm, me2, flags, s);
   const mea::Program& G = P->prog;
-  int H = (hm == MEA_HEL_SUM_NONZERO) ? G.n_hel : (hm == MEA_HEL_SUM_ALL ? (1 << G.n_ext) : 1);
+  int H = (hm == MEA_HEL_SUM_NONZERO) ? P->lanes.n : (hm == MEA_HEL_SUM_ALL ? (1 << G.n_ext) : 1);
   bool fp64 = prec == MEA_PREC_FP64;
   mea::AmpConfig c = mea::cached_plan(P, P->dev, fp64, false, H, n);
   const int ti = fp64 ? 1 : 0;
@@ -353,6 +354,7 @@ mea_status do_evaluate(mea_process_s* P, mea::EvalScratch& S, const double* mom,
   a.n_events = n;
   a.hel_given = hel;
   a.hel_mode = (int)hm;
+  a.paired = P->lanes.paired && hm == MEA_HEL_SUM_NONZERO;
   a.me2 = me2;
   a.flags = flags;
   a.flag_threshold = (float)P->opts.flag_threshold;
@@ -416,7 +418,7 @@ mea_status evaluate_with(mea_process_s* P, EvalScratch& S, const double* mom, in
 
 size_t scratch_estimate(mea_process_s* P, int64_t n, mea_prec_mode prec) {
   const Program& G = P->prog;
-  const int H = G.n_hel;
+  const int H = P->lanes.n;
   const bool fp64 = prec == MEA_PREC_FP64;
   auto work = [&](const DevProgram& d, bool f64, int64_t ne) {
     AmpConfig c = plan_amp(d, f64, H, ne, P->num_sms, P->smem_optin, P->smem_per_sm);
@@ -482,6 +484,7 @@ mea_status mea_create_process(const int* pdg, int n_ext, const mea_options* opts
     destroy(P);
     return fail(MEA_E_UNSUPPORTED, std::string("mea_create_process: ") + e.what());
   }
+  P->lanes = mea::helicity_lanes(P->prog);
   try {
     P->hs = mea::build_helicity_shared(P->prog, P->prog.n_hel);
     P->hs_ok = true;
@@ -529,7 +532,7 @@ mea_status mea_create_process(const int* pdg, int n_ext, const mea_options* opts
   const double* dcfd;
   if ((e = upload(P, G.ops, &dops)) != cudaSuccess || (e = upload(P, G.col, &dcol)) != cudaSuccess ||
       (e = upload(P, G.masks, &dmask)) != cudaSuccess || (e = upload(P, leg, &dleg)) != cudaSuccess ||
-      (e = upload(P, G.hel, &dhel)) != cudaSuccess || (e = upload(P, G.hel_all, &dhall)) != cudaSuccess ||
+      (e = upload(P, P->lanes.hel, &dhel)) != cudaSuccess || (e = upload(P, G.hel_all, &dhall)) != cudaSuccess ||
       (e = upload(P, cff, &dcff)) != cudaSuccess || (e = upload(P, cfd, &dcfd)) != cudaSuccess) {
     destroy(P);
     return fail(e == cudaErrorMemoryAllocation ? MEA_E_NOMEM : MEA_E_CUDA,
@@ -548,7 +551,7 @@ mea_status mea_create_process(const int* pdg, int n_ext, const mea_options* opts
   D.cf_d = dcfd;
   D.cf_inv_den = 1.0 / (double)G.cf_den;
   D.hel = dhel;
-  D.n_hel = G.n_hel;
+  D.n_hel = P->lanes.n;
   D.hel_all = dhall;
   D.g = std::sqrt(4.0 * M_PI * P->opts.alpha_s);
   D.gen = (P->opts.colour_mode == 2) ? nullptr : mea::find_generated(pdg, n_ext);
@@ -598,7 +601,8 @@ mea_status mea_create_process(const int* pdg, int n_ext, const mea_options* opts
     // phased layout for the tensor-core path's amplitude stage; processes it
     // does not cover (and helicity_sharing 1..4) take the kernels below
     try {
-      P->ph = mea::build_phased(G, P->jmap.weight, P->jmap.row, mea::phased_max_area(G, P->smem_optin));
+      P->ph = mea::build_phased(G, P->lanes, P->jmap.weight, P->jmap.row,
+                                mea::phased_max_area(G, P->lanes.n, P->smem_optin));
       phased = true;
     } catch (std::exception&) {
     }
@@ -1027,8 +1031,7 @@ mea_status mea_evaluate_noalloc(mea_process_t P, const double* mom, int64_t n, m
     }
     base = slot.ptr;
   }
-  const mea::Program& G = P->prog;
-  const int H = G.n_hel;
+  const int H = P->lanes.n;
   const bool fp64 = prec == MEA_PREC_FP64;
   const bool reeval = !fp64 && P->opts.reeval_fp64;
   const int ti = fp64 ? 1 : 0;
@@ -1068,6 +1071,7 @@ mea_status mea_evaluate_noalloc(mea_process_t P, const double* mom, int64_t n, m
   a.mom = mom;
   a.n_events = n;
   a.hel_mode = 0;
+  a.paired = P->lanes.paired;
   a.me2 = me2;
   a.flags = flags;
   a.flag_threshold = (float)P->opts.flag_threshold;

@@ -71,7 +71,7 @@ mea_status autotune_locked(mea_process_s* P, const double* mom, int64_t n, mea_p
   P->auto_tuned[prec == MEA_PREC_FP64 ? 1 : 0] = true;
   const bool fp64 = prec == MEA_PREC_FP64;
   const int ti = fp64 ? 1 : 0;
-  const int H = P->prog.n_hel;
+  const int H = P->lanes.n;
   mea::DevProgram dp = P->dev;
   const bool tc = mea::uses_tensor_path(P, prec, MEA_HEL_SUM_NONZERO);
   mea::DevBuf abuf, rowmax, pairk, evf;
@@ -133,6 +133,7 @@ mea_status autotune_locked(mea_process_s* P, const double* mom, int64_t n, mea_p
     mea::AmpLaunch a;
     a.mom = mom;
     a.n_events = n;
+    a.paired = P->lanes.paired;
     a.me2 = me2;
     a.flag_threshold = (float)P->opts.flag_threshold;
     if (tc) {

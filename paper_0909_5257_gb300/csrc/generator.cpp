@@ -1254,4 +1254,24 @@ int count_unique_colour_values(const Program& p) {
   return (int)v.size();
 }
 
+HelLanes helicity_lanes(const Program& p) {
+  HelLanes L;
+  const int H = p.n_hel, n = p.n_ext;
+  L.paired = p.family == FAM_GLUON && H % 2 == 0;
+  for (int h = 0; h < H && L.paired; ++h)
+    for (int l = 0; l < n; ++l)
+      if (p.hel[(size_t)h * n + l] != -p.hel[(size_t)(H - 1 - h) * n + l]) L.paired = false;
+  if (!L.paired) {
+    L.n = H;
+    L.hel = p.hel;
+    return L;
+  }
+  L.n = H / 2;
+  for (int k = 0; k < L.n; ++k) {
+    const int h = p.hel[(size_t)k * n] < 0 ? k : H - 1 - k;
+    L.hel.insert(L.hel.end(), p.hel.begin() + (size_t)h * n, p.hel.begin() + (size_t)(h + 1) * n);
+  }
+  return L;
+}
+
 }  // namespace mea

@@ -45,7 +45,7 @@ struct DevProgram {
   const float* cf_f = nullptr;        // K as float [m*m]
   const double* cf_d = nullptr;       // K as double [m*m]
   double cf_inv_den = 0;              // 1 / D
-  const int8_t* hel = nullptr;        // [n_hel][n_ext] helicities summed in MEA_HEL_SUM_NONZERO
+  const int8_t* hel = nullptr;        // [n_hel][n_ext] lanes of MEA_HEL_SUM_NONZERO (generator.h, HelLanes)
   int n_hel = 0;
   const int8_t* hel_all = nullptr;    // [2^n_ext][n_ext]
   double g = 0;                       // g_s
@@ -89,6 +89,7 @@ struct AmpLaunch {
   const int32_t* event_list = nullptr;  // optional: evaluate mom[event_list[i]] for i < *list_count
   const int32_t* list_count = nullptr;  // device count for event_list mode
   const int8_t* hel_given = nullptr;  // [n_events][n_ext] for one given helicity per event
+  bool paired = false;                // the helicity sum reads every lane twice (HelLanes)
   int hel_mode = 0;                   // 0 nonzero set, 1 all 2^n, 2 given
   double* me2 = nullptr;
   uint8_t* flags = nullptr;
@@ -163,7 +164,7 @@ cudaError_t launch_amp_hsp(const DevProgram& p, const AmpConfig& c, const AmpLau
 // Phased kernel: every stored wavefunction in shared memory, a CTA per event.
 constexpr int64_t kPhasedMaxLda = 0x3fffffff;
 bool phased_supported(const DevProgram& p, bool fp64, int H);
-int phased_max_area(const Program& P, size_t max_smem);  // variants that fit a CTA's shared memory
+int phased_max_area(const Program& P, int H, size_t max_smem);  // variants that fit a CTA's shared memory
 std::vector<AmpConfig> phased_candidates(const DevProgram& p, int H, int64_t n_events, int num_sms, size_t max_smem,
                                          size_t smem_per_sm);
 const AmpConfig* phased_default(const std::vector<AmpConfig>& cands);  // the untuned shape

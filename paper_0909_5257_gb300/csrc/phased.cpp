@@ -50,9 +50,9 @@ void check(bool ok, const char* why) {
 
 }  // namespace
 
-PhProgram build_phased(const Program& P, const std::vector<float>& weight,
+PhProgram build_phased(const Program& P, const HelLanes& lanes, const std::vector<float>& weight,
                        const std::vector<int>& row, int max_area) {
-  const int n = P.n_ext, H = P.n_hel;
+  const int n = P.n_ext, H = lanes.n;
   check(n >= 6 && n <= 7, "6 or 7 legs");
   check(H >= 1 && H <= 128, "at most 128 combinations");
   check(P.masks.size() <= 256, "at most 256 event-table rows");
@@ -64,7 +64,7 @@ PhProgram build_phased(const Program& P, const std::vector<float>& weight,
   std::vector<uint32_t> hbits(H, 0);
   for (int h = 0; h < H; ++h)
     for (int l = 0; l < n; ++l)
-      if (P.hel[(size_t)h * n + l] > 0) hbits[h] |= 1u << l;
+      if (lanes.hel[(size_t)h * n + l] > 0) hbits[h] |= 1u << l;
   Q.hv.assign((size_t)128 << n, 0);
   for (uint32_t S = 0; S <= all; ++S)
     for (int h = 0; h < H; ++h) Q.hv[S * 128 + h] = (uint8_t)pext8(hbits[h], S);

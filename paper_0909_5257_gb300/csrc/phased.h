@@ -115,10 +115,10 @@ struct PhProgram {
   double cost = 0;                 // estimated warp instructions per event
 };
 
-// weight[d]: sum of the colour coefficients' magnitudes of diagram d
+// lanes: the helicity combinations; weight[d]: sum of the colour coefficients' magnitudes of diagram d
 // (JampMap::weight), row[d] its row in the amplitude buffer (JampMap::row).  Throws std::runtime_error when the program does not have
 // the structure above or its area exceeds max_area variants.
-PhProgram build_phased(const Program& P, const std::vector<float>& weight,
+PhProgram build_phased(const Program& P, const HelLanes& lanes, const std::vector<float>& weight,
                        const std::vector<int>& row, int max_area);
 
 }  // namespace mea

@@ -55,6 +55,7 @@ mea_status set_error(mea_status s, const std::string& msg);
 
 struct mea_process_s {
   mea::Program prog;
+  mea::HelLanes lanes;  // evaluated combinations of the non-vanishing helicity sum
   mea::HsProgram hs;  // helicity-shared layout of prog (valid when hs_ok)
   bool hs_ok = false;
   mea::HsSplitProgram hsp;  // split layout of prog (valid when hsp_ok)

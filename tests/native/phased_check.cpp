@@ -69,7 +69,8 @@ int main(int argc, char** argv) {
       p = e + 1;
     }
     const Program P = build_program(pdg);
-    const int n = P.n_ext, H = P.n_hel;
+    const HelLanes lanes = helicity_lanes(P);
+    const int n = P.n_ext, H = lanes.n;
     std::vector<float> weight(P.n_diagrams);
     for (int d = 0; d < P.n_diagrams; ++d) weight[d] = 1.f + (float)(d % 7);
     std::vector<int> row_of(P.n_diagrams), row(P.n_diagrams);  // a permutation
@@ -77,7 +78,7 @@ int main(int argc, char** argv) {
     if (P.n_diagrams % 5 == 0)
       for (int d = 0; d < P.n_diagrams; ++d) row[d] = P.n_diagrams - 1 - d;
     for (int d = 0; d < P.n_diagrams; ++d) row_of[row[d]] = d;
-    const PhProgram Q = build_phased(P, weight, row, 6800);
+    const PhProgram Q = build_phased(P, lanes, weight, row, 6800);
 
     std::mt19937_64 rng(0x5eed + a);
     auto u = [&]() { return std::uniform_real_distribution<double>(-1.0, 1.0)(rng); };
@@ -114,7 +115,7 @@ int main(int argc, char** argv) {
         if (is_amp_op(op.type))
           ref[(size_t)h * P.n_diagrams + d++] = closed(op.type, op.leg, x, mrow(op.min[0]), mrow(op.min[1]), mrow(op.min[2]));
         else if (op.type == OP_EXT)
-          slots[op.out] = in.ext[op.leg][P.hel[(size_t)h * n + op.leg] > 0];
+          slots[op.out] = in.ext[op.leg][lanes.hel[(size_t)h * n + op.leg] > 0];
         else
           slots[op.out] = made(op.type, op.leg, x, mrow(op.min[0]), mrow(op.min[1]), mrow(op.min[2]), mrow(op.mout));
       }
