@@ -63,7 +63,13 @@ __device__ void prep_leg(const DevProgram& P, const double* mom, int k, R* et) {
   if (type == 0) {
     R kt = sqrt(kt2);
     R ct, st, cp, sp;
-    if (kt > R(0)) { ct = pz / kk; st = kt / kk; cp = px / kt; sp = py / kt; }
+    if constexpr (std::is_same<R, double>::value) {
+      // two reciprocal roots instead of two roots and four divisions (the FP64
+      // pipe is what bounds the FP64 path)
+      const double rk = rsqrt(kt2 + pz * pz), rt = rsqrt(kt2);
+      if (kt2 > 0.0) { ct = pz * rk; st = kt2 * rt * rk; cp = px * rt; sp = py * rt; }
+      else { ct = pz < 0.0 ? -1.0 : 1.0; st = 0.0; cp = 1.0; sp = 0.0; }
+    } else if (kt > R(0)) { ct = pz / kk; st = kt / kk; cp = px / kt; sp = py / kt; }
     else { ct = pz < R(0) ? R(-1) : R(1); st = R(0); cp = R(1); sp = R(0); }
     o[0] = ct * cp; o[1] = ct * sp; o[2] = -st;
     o[3] = -sp; o[4] = cp; o[5] = R(0);

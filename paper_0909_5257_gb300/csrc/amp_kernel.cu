@@ -574,6 +574,15 @@ static int interp_resident(bool fp64, bool jsm, bool ssm, bool aout, int threads
 
 AmpConfig plan_amp(const DevProgram& p, bool fp64, int H, int64_t n_events, int num_sms,
                    size_t max_smem, size_t smem_per_sm, int hint) {
+  if (hint == 0 && ordered_supported(p, fp64, H)) {
+    const std::vector<AmpConfig> cs = ordered_candidates(p, H, num_sms, max_smem, smem_per_sm);
+    if (!cs.empty()) {
+      AmpConfig c = *ordered_default(cs);
+      const int64_t tiles = (n_events + c.E_cta - 1) / c.E_cta;
+      if (tiles < c.grid) c.grid = (int)std::max<int64_t>(tiles, 1);
+      return c;
+    }
+  }
   if (p.gen && hint == 0) return plan_generated(p, fp64, H, n_events, num_sms);
   if (hint == 0 && phased_supported(p, fp64, H)) {
     const std::vector<AmpConfig> cs = phased_candidates(p, H, n_events, num_sms, max_smem, smem_per_sm);
@@ -670,6 +679,9 @@ std::vector<AmpConfig> candidate_configs(const DevProgram& p, bool fp64, int H, 
     if (tiles < c.grid) c.grid = (int)std::max<int64_t>(tiles, 1);
     return c;
   };
+  if (ordered_supported(p, fp64, H))
+    for (AmpConfig c : ordered_candidates(p, H, num_sms, max_smem, smem_per_sm)) out.push_back(cap(c));
+  if (!out.empty()) return out;
   if (p.gen) {
     // FP64: one variant; FP32: every register cap, each with its body (see
     // gen_body_variant)
@@ -764,6 +776,7 @@ std::vector<AmpConfig> candidate_configs(const DevProgram& p, bool fp64, int H, 
 }
 
 size_t jamp_scratch_bytes_needed(const DevProgram& p, bool fp64, const AmpConfig& c) {
+  if (c.ordered) return ordered_amp_bytes(p, c);
   if (c.jamp_in_smem) return 0;
   const int JW = fp64 ? 2 : 4;
   return (size_t)c.grid * p.n_colour * JW * c.threads * (fp64 ? sizeof(double) : sizeof(float));
@@ -772,6 +785,7 @@ size_t jamp_scratch_bytes_needed(const DevProgram& p, bool fp64, const AmpConfig
 size_t slot_scratch_bytes_needed(const DevProgram& p, bool fp64, const AmpConfig& c) {
   if (c.helshare) return hs_arena_bytes(p, c);
   if (c.hsplit) return hsp_area_bytes(p, c);
+  if (c.ordered) return ordered_area_bytes(p, c);
   if (c.slots_in_smem || c.phased) return 0;
   return (size_t)c.grid * p.n_slots * 8 * c.threads * (fp64 ? sizeof(double) : sizeof(float));
 }
@@ -805,6 +819,12 @@ cudaError_t launch_amp(const DevProgram& p, bool fp64, const AmpConfig& c, const
                        cudaStream_t s) {
   if (c.grid <= 0) return cudaSuccess;
   cudaError_t err = cudaSuccess;
+  if (c.ordered) {
+    if (!fp64) return cudaErrorInvalidValue;
+    err = launch_ordered(p, c, a, s);
+    if (err == cudaSuccess) ++launch_counter();
+    return err;
+  }
   if (c.phased) {
     if (fp64) return cudaErrorInvalidValue;
     err = launch_amp_phased(p, c, a, s);

@@ -23,6 +23,7 @@
 #include "jamp_gemm.h"
 #include "generator.h"
 #include "kernels.h"
+#include "ordered.h"
 #include "phased.h"
 #include "process.h"
 
@@ -596,6 +597,32 @@ mea_status mea_create_process(const int* pdg, int n_ext, const mea_options* opts
       std::vector<__half>().swap(P->jmap.tiles);
     }
   }
+  try {
+    // FP64 path: the ordered recursion; where it does not apply the kernels of
+    // the diagram program stay
+    if (G.family == mea::FAM_GLUON && n_ext == 4) throw std::runtime_error("straight-line kernel");  // ordered_kernel.cu
+    mea::OrdProgram O = mea::build_ordered(G);
+    std::vector<uint8_t> bar(O.stages.size(), 1);
+    for (size_t k = 0; k + 1 < O.stages.size(); ++k) bar[k] = O.level[k + 1] != O.level[k] ? 1 : 0;
+    for (int a = 0; a < O.n_colour; ++a)
+      for (int b = a + 1; b < O.n_colour; ++b) O.kmat[(size_t)a * O.n_colour + b] *= 2.0;
+    const mea::OrdStage* ds = nullptr;
+    if ((e = upload(P, O.stages, &ds)) != cudaSuccess || (e = upload(P, bar, &D.ord_barrier)) != cudaSuccess ||
+        (e = upload(P, O.rec, &D.ord_rec)) != cudaSuccess || (e = upload(P, O.fidx, &D.ord_fidx)) != cudaSuccess ||
+        (e = upload(P, O.range, &D.ord_range)) != cudaSuccess || (e = upload(P, O.kmat, &D.ord_k)) != cudaSuccess) {
+      destroy(P);
+      return fail(e == cudaErrorMemoryAllocation ? MEA_E_NOMEM : MEA_E_CUDA, std::string("mea_create_process: ") + cudaGetErrorString(e));
+    }
+    D.ord_n_stages = (int)O.stages.size();
+    D.ord_colour = O.n_colour;
+    D.ord_H = O.H;
+    D.ord_area = O.area;
+    D.ord_nf = O.n_f;
+    D.ord_norm = O.norm * std::pow(D.g, 2 * n_ext - 4);
+    D.ord_lanes = P->lanes.n;
+    D.ord_stages = ds;
+  } catch (std::exception&) {
+  }
   bool phased = false;
   if (P->jmap.ok && P->opts.helicity_sharing == 0) {
     // phased layout for the tensor-core path's amplitude stage; processes it
@@ -1053,6 +1080,13 @@ mea_status mea_evaluate_noalloc(mea_process_t P, const double* mom, int64_t n, m
   const size_t list_off = 256;
   const size_t list_bytes = reeval ? (((size_t)n * sizeof(int32_t) + 255) & ~size_t(255)) : 0;
   const size_t work_off = list_off + list_bytes;
+  // the ordered recursion keeps an event's currents per CTA: as many CTAs as the array holds
+  for (mea::AmpConfig* q : {&c, &c2})
+    if (q->ordered && work_off < (size_t)MEA_NOALLOC_SCRATCH_BYTES) {
+      const size_t room = (size_t)MEA_NOALLOC_SCRATCH_BYTES - work_off - 512;
+      const size_t per = (work_bytes(true, *q) + q->grid - 1) / q->grid;
+      if (per > 0) q->grid = (int)std::max<size_t>(1, std::min<size_t>((size_t)q->grid, room / per));
+    }
   size_t work = work_bytes(fp64, c);
   if (reeval) work = std::max(work, work_bytes(true, c2));
   const size_t need = work_off + work;

@@ -884,6 +884,7 @@ Program build_program(const std::vector<int>& pdg, const BuildOptions& opt) {
   if (B.amps.empty()) throw std::runtime_error("process has no tree diagrams");
   P.n_diagrams = (int)B.amps.size();
   P.n_colour = B.n_colour;
+  P.basis = B.basis_chains;
 
   // ---- vertex partials.  Every amplitude vertex is linear in each input; an
   // amplitude whose vertex shares all inputs but one with other amplitudes

@@ -17,8 +17,10 @@
 //     shared partial vertex (heget.cuh, "vertex partials");
 //   * an evaluation order with wavefunction-slot reuse.
 #pragma once
+#include <array>
 #include <cstdint>
 #include <string>
+#include <utility>
 #include <vector>
 
 namespace mea {
@@ -102,6 +104,9 @@ struct Program {
   std::vector<int8_t> hel_all;        // [2^n_ext][n_ext]
   double flops_per_hel = 0;
   double flops_per_hel_plain = 0;     // the same with one vertex call per diagram
+  // colour basis: per vector its strings of gluon labels (100: exchanged gluon)
+  // and their ends (row, column legs; -1, -1: a trace that starts with the root)
+  std::vector<std::vector<std::pair<std::vector<int>, std::array<int, 2>>>> basis;
   std::string basis_text;             // human-readable basis (debug)
 };
 

@@ -47,6 +47,7 @@
 #include <cstdlib>
 #include <numeric>
 
+#include "colour_base.h"
 #include "jamp_gemm.h"
 #include "kernels.h"
 #include "tc_common.cuh"
@@ -458,74 +459,6 @@ __global__ void __launch_bounds__(kThreads, 1) jamp_gemm_kernel(JampGemmArgs g) 
   if (warp == 0) tmem_dealloc(tmem, tmem_cols);
 }
 
-// Base of the rows of C (m x kd small integers): the first rows that no
-// earlier ones generate, and the others as sums of them, by elimination
-// modulo a prime on random combinations of the columns; the result is checked
-// exactly by the caller.  Returns false unless the base is rows 0 .. mb - 1
-// and every coefficient is 0, 1 or -1.
-bool find_base(const std::vector<int>& C, int m, int kd, int& mb, std::vector<std::vector<int>>& coef) {
-  typedef unsigned long long u64;
-  const u64 P = 2147483647ull;
-  auto inv = [&](u64 a) {
-    u64 r = 1, e = P - 2;
-    for (; e; e >>= 1, a = a * a % P)
-      if (e & 1) r = r * a % P;
-    return r;
-  };
-  const int cols = m + 8;
-  u64 seed = 0x9E3779B97F4A7C15ull;
-  std::vector<u64> X((size_t)m * cols, 0), rnd(cols);
-  for (int d = 0; d < kd; ++d) {
-    for (u64& x : rnd) {  // a linear congruential sequence
-      seed = seed * 6364136223846793005ull + 1442695040888963407ull;
-      x = (seed >> 33) % P;
-    }
-    for (int a = 0; a < m; ++a) {
-      const int c = C[(size_t)a * kd + d];
-      if (!c) continue;
-      const u64 cc = (u64)((c + (long long)P) % (long long)P);
-      for (int j = 0; j < cols; ++j) X[(size_t)a * cols + j] = (X[(size_t)a * cols + j] + cc * rnd[j]) % P;
-    }
-  }
-  std::vector<std::vector<u64>> B, T;  // reduced rows and what they are of the base rows
-  std::vector<int> piv;
-  mb = 0;
-  coef.clear();
-  for (int a = 0; a < m; ++a) {
-    std::vector<u64> r(X.begin() + (size_t)a * cols, X.begin() + (size_t)(a + 1) * cols), c(m, 0);
-    for (size_t b = 0; b < B.size(); ++b) {
-      const u64 f = r[piv[b]];
-      if (!f) continue;
-      for (int j = 0; j < cols; ++j) r[j] = (r[j] + (P - f) * B[b][j]) % P;
-      for (int j = 0; j < mb; ++j) c[j] = (c[j] + f * T[b][j]) % P;
-    }
-    int q = -1;
-    for (int j = 0; j < cols && q < 0; ++j)
-      if (r[j]) q = j;
-    if (q >= 0) {
-      if (a != mb) return false;  // the base is not a prefix
-      const u64 iv = inv(r[q]);
-      for (u64& x : r) x = x * iv % P;
-      std::vector<u64> tb(m, 0);
-      for (int j = 0; j < mb; ++j) tb[j] = (P - c[j]) % P * iv % P;
-      tb[mb] = iv;
-      B.push_back(r);
-      T.push_back(tb);
-      piv.push_back(q);
-      ++mb;
-    } else {
-      std::vector<int> k(m, 0);
-      for (int j = 0; j < mb; ++j) {
-        if (c[j] == 1) k[j] = 1;
-        else if (c[j] == P - 1) k[j] = -1;
-        else if (c[j] != 0) return false;
-      }
-      coef.push_back(k);
-    }
-  }
-  return true;
-}
-
 }  // namespace
 
 JampMap build_jamp_map(const Program& p) {
@@ -568,33 +501,12 @@ JampMap build_jamp_map(const Program& p) {
 
   // base columns: one block of them, their terms and a 64-row stage of their
   // integers must fit (kMaxNC columns do)
+  const ColourBase base = find_colour_base(p);
   M.mb = M.m;
-  {
-    int mb = 0;
-    std::vector<std::vector<int>> coef;
-    if (find_base(C, M.m, kd, mb, coef) && mb < M.m && mb <= kMaxNC) {
-      bool exact = true;
-      std::vector<uint16_t> index, term;
-      for (int a = mb; a < M.m && exact; ++a) {
-        const std::vector<int>& k = coef[a - mb];
-        std::vector<int> row(kd, 0);
-        index.push_back((uint16_t)term.size());
-        for (int sg : {1, -1}) {
-          for (int b = 0; b < mb; ++b)
-            if (k[b] == sg) {
-              term.push_back((uint16_t)b);
-              for (int x = 0; x < kd; ++x) row[x] += sg * C[(size_t)b * kd + x];
-            }
-          index.push_back((uint16_t)term.size());
-        }
-        exact = std::equal(row.begin(), row.end(), C.begin() + (size_t)a * kd);
-      }
-      if (exact && term.size() <= 4096) {
-        M.mb = mb;
-        M.kk_index = index;
-        M.kk_term = term;
-      }
-    }
+  if (base.mb < M.m && base.mb <= kMaxNC && base.term.size() <= 4096) {
+    M.mb = base.mb;
+    M.kk_index = base.index;
+    M.kk_term = base.term;
   }
   M.nc = std::min(kMaxNC, ((M.mb + 15) / 16) * 16);
   M.n_splits = (M.mb + M.nc - 1) / M.nc;

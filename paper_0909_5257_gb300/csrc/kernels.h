@@ -13,6 +13,7 @@ struct DevProgram;
 struct AmpConfig;
 struct AmpLaunch;
 struct HsOp;
+struct OrdStage;
 struct PhUnit;
 struct PhSet;
 
@@ -76,6 +77,18 @@ struct DevProgram {
   int ph_phases = 0;
   int ph_area = 0;
   int ph_H = 0;
+  // ordered recursion (ordered.h, FP64 path), or null: stages, whether a barrier
+  // follows each, records, amplitude of (ordering, combination), orderings of
+  // each combination, colour matrix (upper triangle, off-diagonal doubled)
+  const OrdStage* ord_stages = nullptr;
+  const uint8_t* ord_barrier = nullptr;
+  const uint64_t* ord_rec = nullptr;
+  const uint16_t* ord_fidx = nullptr;
+  const int* ord_range = nullptr;
+  const double* ord_k = nullptr;
+  int ord_n_stages = 0, ord_colour = 0, ord_H = 0, ord_area = 0, ord_nf = 0;
+  int ord_lanes = 0;                    // the H that plans of the non-vanishing helicity sum carry
+  double ord_norm = 0;                  // OrdProgram::norm g^(2n-4)
   // per op: bits 0..3 input k is the previous op's output, bit 4 the op's
   // output is read only by the next op (amplitude-output interpreter with
   // register forwarding), or null
@@ -120,6 +133,8 @@ struct AmpConfig {
   bool fwd = false;       // amplitude-output interpreter: the previous op's output forwarded in registers
   bool hsplit = false;    // amplitude-output mode: the split kernel (amp_hsp_kernel, amp_hs_kernel.cu):
                           // E_cta events x H lanes; slots_in_smem = its prologue area in shared memory
+  bool ordered = false;   // FP64: the ordered recursion (ordered_kernel.cu), tiles of E_cta events;
+                          // slots_in_smem its currents, jamp_in_smem its amplitudes in shared memory
   bool phased = false;    // amplitude-output mode: the phased kernel (amp_phased_kernel.cu), a CTA per event
   bool helshare = false;  // amplitude-output mode: the helicity-shared kernel (amp_hs_kernel.cu):
                           // one warp per event, E_cta = warps per CTA, regvar its register
@@ -160,6 +175,14 @@ size_t hsp_smem_bytes(const DevProgram& p, int events, bool area_in_smem);
 size_t hsp_area_bytes(const DevProgram& p, const AmpConfig& c);
 std::vector<AmpConfig> hsp_candidates(const DevProgram& p, int H, int num_sms, size_t max_smem, size_t smem_per_sm);
 cudaError_t launch_amp_hsp(const DevProgram& p, const AmpConfig& c, const AmpLaunch& a, cudaStream_t s);
+
+// Ordered recursion (FP64, the non-vanishing helicity sum).
+bool ordered_supported(const DevProgram& p, bool fp64, int H);
+std::vector<AmpConfig> ordered_candidates(const DevProgram& p, int H, int num_sms, size_t max_smem, size_t smem_per_sm);
+const AmpConfig* ordered_default(const std::vector<AmpConfig>& cands);  // the untuned shape
+size_t ordered_area_bytes(const DevProgram& p, const AmpConfig& c);     // global memory of a launch
+size_t ordered_amp_bytes(const DevProgram& p, const AmpConfig& c);
+cudaError_t launch_ordered(const DevProgram& p, const AmpConfig& c, const AmpLaunch& a, cudaStream_t s);
 
 // Phased kernel: every stored wavefunction in shared memory, a CTA per event.
 constexpr int64_t kPhasedMaxLda = 0x3fffffff;
