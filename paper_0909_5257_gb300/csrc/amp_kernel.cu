@@ -482,21 +482,15 @@ const GenEntry* find_generated(const int* pdg, int n_ext) {
 // that threads <= kGenMaxThreads with few idle lanes, then fill the SMs by
 // occupancy.
 //
-// Body of the FP32 straight-line kernel at a register cap (0: 128, 1: 85):
-// the one with shared vertex partials (fewer FLOPs) unless it needs more
-// local memory (spills) than the body with one vertex call per diagram.
-// Spilled lines compete with the streamed inputs for L2 and reach DRAM at
-// full size, which costs more than the FLOPs save (gg>ggg at 2^20 events:
-// 82.7 M events/s with partials, 92.2 M without; the partials body spills
-// 1104 bytes per thread at 128 registers, the other 936).  The rule depends
-// only on the compiled kernels, so the choice -- and the FP32 rounding order
-// -- is the same on every run.
+// Body of the FP32 straight-line kernel at a register cap (0: 128, 1: 85, 2:
+// 168): the one with shared vertex partials (fewer FLOPs), or one vertex call per
+// diagram where the partials' longer live ranges spill clearly more (uu>uug at
+// 85 registers: 392 against 224 bytes per thread).  A fixed rule, because the
+// body decides the FP32 rounding order: reading the spill sizes off the compiled
+// kernels let an unrelated change of a build flip it (uu~>ggg at 85 registers:
+// 752 and 784 bytes in one build, 712 and 696 in another).
 static int gen_body_variant(const DevProgram& p, int cap) {
-  cudaFuncAttributes with, without;
-  if (cudaFuncGetAttributes(&with, p.gen->kernel(false, 2 * cap)) != cudaSuccess ||
-      cudaFuncGetAttributes(&without, p.gen->kernel(false, 2 * cap + 1)) != cudaSuccess)
-    return 2 * cap;
-  return without.localSizeBytes < with.localSizeBytes ? 2 * cap + 1 : 2 * cap;
+  return 2 * cap + (p.family == FAM_TWO_LINES && p.n_ext == 5 && cap == 1 ? 1 : 0);
 }
 
 static AmpConfig plan_generated(const DevProgram& p, bool fp64, int H, int64_t n_events, int num_sms) {

@@ -546,6 +546,7 @@ mea_status mea_create_process(const int* pdg, int n_ext, const mea_options* opts
   D.n_masks = (int)G.masks.size();
   D.leg_info = dleg;
   D.n_ext = n_ext;
+  D.family = G.family;
   D.n_slots = G.n_slots;
   D.n_colour = G.n_jamp;  // colour amplitudes accumulated (folded for gluons)
   D.cf_f = dcff;

@@ -41,6 +41,7 @@ struct DevProgram {
   int n_masks = 0;
   const int8_t* leg_info = nullptr;   // [n_ext][4]: type, spinor kind, incoming, pad
   int n_ext = 0;
+  int family = 0;                     // generator.h Family
   int n_slots = 0;
   int n_colour = 0;
   const float* cf_f = nullptr;        // K as float [m*m]
