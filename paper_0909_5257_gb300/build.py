@@ -67,7 +67,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     # 1. emit the straight-line per-process kernels with the generator
     tool = os.path.join(BUILD_DIR, "mea_codegen")
     r = subprocess.run(["g++", "-O2", "-std=c++17", "-fopenmp", "-o", tool, os.path.join(CSRC, "codegen.cpp"),
-                        os.path.join(CSRC, "generator.cpp")], capture_output=True, text=True)
+                        os.path.join(CSRC, "colour_base.cpp"), os.path.join(CSRC, "generator.cpp")], capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"codegen tool build failed:\n{r.stderr}")
     gen_dir = os.path.join(BUILD_DIR, "generated")

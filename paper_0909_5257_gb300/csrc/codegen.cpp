@@ -18,6 +18,7 @@
 #include <string>
 #include <vector>
 
+#include "colour_base.h"
 #include "generator.h"
 
 namespace {
@@ -50,8 +51,11 @@ void emit_body(std::ostringstream& o, const mea::Program& P, const std::string& 
   o << "  __device__ __forceinline__ static void run(const R* __restrict__ et, const R* __restrict__ mt,\n"
        "                                             uint32_t lam, R g, R gg, double inv_den, double& val,\n"
        "                                             float& kappa) {\n";
-  o << "    cx<R> J[" << m << "];\n    cx<R> Jl[" << m << "];\n";
-  o << "#pragma unroll\n    for (int a = 0; a < " << m << "; ++a) { J[a] = mk<R>(R(0), R(0)); Jl[a] = J[a]; }\n";
+  // Only the base of the colour amplitudes is accumulated (colour_base.h: half of
+  // them for pure gluons); the others are sums of its compensated sums at the
+  // end -- half the additions and half the registers.
+  const ColourBase base = find_colour_base(P);
+  o << "    JSum<R> J[" << m << "];\n";
   o << "    float mass = 0.f;\n";
   // Common factor of the colour coefficients: the amplitudes are accumulated
   // with the cofactors (+-1 for every process here) and J is scaled by the
@@ -134,16 +138,15 @@ void emit_body(std::ostringstream& o, const mea::Program& P, const std::string& 
         for (uint32_t k = 0; k < op.col_count; ++k) {
           const ColEntry& c = P.col[op.col_begin + k];
           wsum += std::abs((int)c.re) + std::abs((int)c.im);
+          if ((int)c.alpha >= base.mb) continue;
           if (cfac_real) {
             const int n = (int)c.re / cfac;
             if (n == 1 || n == -1)
-              o << "      jadd<R>(J[" << c.alpha << "], Jl[" << c.alpha << "], " << (n > 0 ? "a" : "neg<R>(a)")
-                << ");\n";
+              o << "      jadd(J[" << c.alpha << "], " << (n > 0 ? "a" : "neg<R>(a)") << ");\n";
             else
-              o << "      jadd<R>(J[" << c.alpha << "], Jl[" << c.alpha << "], mk<R>(R(" << n << ") * a.r, R(" << n
-                << ") * a.i));\n";
+              o << "      jadd(J[" << c.alpha << "], mk<R>(R(" << n << ") * a.r, R(" << n << ") * a.i));\n";
           } else {
-            o << "      jadd<R>(J[" << c.alpha << "], Jl[" << c.alpha << "], mk<R>(R(" << (int)c.re << ") * a.r - R("
+            o << "      jadd(J[" << c.alpha << "], mk<R>(R(" << (int)c.re << ") * a.r - R("
               << (int)c.im << ") * a.i, R(" << (int)c.re << ") * a.i + R(" << (int)c.im << ") * a.r));\n";
           }
         }
@@ -157,10 +160,15 @@ void emit_body(std::ostringstream& o, const mea::Program& P, const std::string& 
     }
     if (!is_amp_op(op.type)) slot_op[op.out] = (int)i;
   }
+  for (int a = base.mb; a < m; ++a) {
+    const uint16_t* ix = &base.index[3 * (a - base.mb)];
+    for (int k = ix[0]; k < ix[2]; ++k)
+      o << "    " << (k < ix[1] ? "jadd" : "jsub") << "(J[" << a << "], J[" << base.term[k] << "]);\n";
+  }
   // colour quadratic form with the integer colour matrix (symmetric)
   o << "    cx<R> F[" << m << "];\n    float jabs = 0.f;\n";
   const std::string scale = (cfac_real && cfac != 1) ? " * R(" + std::to_string(cfac) + ")" : "";
-  o << "#pragma unroll\n    for (int a = 0; a < " << m << "; ++a) { F[a] = jfin<R>(J[a], Jl[a]); F[a].r = F[a].r"
+  o << "#pragma unroll\n    for (int a = 0; a < " << m << "; ++a) { F[a] = jfin(J[a]); F[a].r = F[a].r"
     << scale << "; F[a].i = F[a].i" << scale << "; jabs += (float)(fabs(F[a].r) + fabs(F[a].i)); }\n";
   o << "    R tot = R(0);\n";
   for (int a = 0; a < m; ++a) {

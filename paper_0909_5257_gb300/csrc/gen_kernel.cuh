@@ -14,67 +14,85 @@ namespace {
 
 constexpr int kGenMaxThreads = 256;
 
-// J += (cr + i ci) a, two-sum compensated in FP32 (lo collects the rounding
-// errors); mass accumulates sum |c a| for the cancellation indicator.
+// A colour amplitude under accumulation: FP64 plain, FP32 two-sum compensated
+// (lo collects the rounding errors) with its real and imaginary parts as one
+// packed pair, so that a compensated addition is 7 instructions instead of 14.
+// The FP32 pipe and the spills of the long body bound these kernels: packed
+// additions together with accumulating the base columns only take 2^20 events
+// of gg>ggg from 6.77 to 4.22 ms (168 registers) and from 8.03 to 5.25 ms
+// (128); gg>gg 0.66 ms either way (compute is not what it waits for).
 template <typename R>
-__device__ __forceinline__ void jacc(cx<R>& hi, cx<R>& lo, float& mass, R cr, R ci, cx<R> a) {
-  R xr = cr * a.r - ci * a.i;
-  R xi = cr * a.i + ci * a.r;
-  if constexpr (std::is_same<R, float>::value) {
-    float s, e;
-    two_sum(hi.r, xr, s, e);
-    hi.r = s;
-    lo.r += e;
-    two_sum(hi.i, xi, s, e);
-    hi.i = s;
-    lo.i += e;
-    mass += fabsf(xr) + fabsf(xi);
-  } else {
-    hi.r += xr;
-    hi.i += xi;
-  }
+struct JSum {
+  cx<R> hi{R(0), R(0)};
+};
+template <>
+struct JSum<float> {
+  unsigned long long hi = 0, lo = 0;
+};
+
+__device__ __forceinline__ unsigned long long jpack(cx<float> a) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.r), "f"(a.i));
+  return r;
+}
+__device__ __forceinline__ cx<float> junpack(unsigned long long v) {
+  cx<float> a;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a.r), "=f"(a.i) : "l"(v));
+  return a;
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long sub2(unsigned long long a, unsigned long long b) {  // a - b, rounded once
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(b), "l"(0xBF800000BF800000ull), "l"(a));
+  return r;
 }
 
-// J += a, two-sum compensated in FP32 (the coefficient is folded into a by
-// the emitter; mass is accumulated once per amplitude).
-template <typename R>
-__device__ __forceinline__ void jadd(cx<R>& hi, cx<R>& lo, cx<R> a) {
-  if constexpr (std::is_same<R, float>::value) {
-    float s, e;
-    two_sum(hi.r, a.r, s, e);
-    hi.r = s;
-    lo.r += e;
-    two_sum(hi.i, a.i, s, e);
-    hi.i = s;
-    lo.i += e;
-  } else {
-    hi.r += a.r;
-    hi.i += a.i;
-  }
+// J += a
+__device__ __forceinline__ void jadd(JSum<float>& J, unsigned long long a) {
+  const unsigned long long s = add2(J.hi, a);
+  const unsigned long long bp = sub2(s, J.hi);
+  const unsigned long long e = add2(sub2(J.hi, sub2(s, bp)), sub2(a, bp));
+  J.hi = s;
+  J.lo = add2(J.lo, e);
 }
+__device__ __forceinline__ void jadd(JSum<float>& J, cx<float> a) { jadd(J, jpack(a)); }
+__device__ __forceinline__ void jadd(JSum<double>& J, cx<double> a) {
+  J.hi.r += a.r;
+  J.hi.i += a.i;
+}
+// J += x, J -= x for another sum x
+__device__ __forceinline__ void jadd(JSum<float>& J, const JSum<float>& x) {
+  jadd(J, x.hi);
+  J.lo = add2(J.lo, x.lo);
+}
+__device__ __forceinline__ void jadd(JSum<double>& J, const JSum<double>& x) { jadd(J, x.hi); }
+__device__ __forceinline__ void jsub(JSum<float>& J, const JSum<float>& x) {
+  jadd(J, x.hi ^ 0x8000000080000000ull);
+  J.lo = sub2(J.lo, x.lo);
+}
+__device__ __forceinline__ void jsub(JSum<double>& J, const JSum<double>& x) { jadd(J, cx<double>{-x.hi.r, -x.hi.i}); }
 
 template <typename R>
 __device__ __forceinline__ cx<R> neg(cx<R> a) {
   return cx<R>{-a.r, -a.i};
 }
 
-template <typename R>
-__device__ __forceinline__ cx<R> jfin(cx<R> hi, cx<R> lo) {
-  if constexpr (std::is_same<R, float>::value) return cx<R>{hi.r + lo.r, hi.i + lo.i};
-  return hi;
-}
+__device__ __forceinline__ cx<float> jfin(const JSum<float>& J) { return junpack(add2(J.hi, J.lo)); }
+__device__ __forceinline__ cx<double> jfin(const JSum<double>& J) { return J.hi; }
 
 // Register-cap variants: MINB resident CTAs of MAXT threads per SM cap a
-// thread at 65536 / (MAXT MINB) registers.  Spilling part of the long
-// straight-line body to L1 in exchange for more resident warps wins for the
-// 3-jet bodies (measured on 2^20 events: gg>ggg 14.4 ms at 255 registers,
-// 11.3 ms at 128; uu>uug 2.6 ms at 128, 2.25 ms at 85), so the FP32 bodies
-// come at 128 (256 threads, MINB 2), 85 (256, 3) and 168 (192, 2) registers --
-// the last halves the gg>ggg spill footprint (640 against 936 bytes per
-// thread) so that it stays in L1 with 10 resident warps -- and the autotuner
-// picks; the FP64 bodies come at 128.  A module that also held uncapped FP32
-// variants measured 25-45 % slower on the same 128-register kernel, so none
-// is built.
+// thread at 65536 / (MAXT MINB) registers.  More registers spill less of the
+// long straight-line body, fewer keep more warps resident, and which wins
+// depends on the body, so the FP32 bodies come at 128 (256 threads, MINB 2),
+// 85 (256, 3) and 168 (192, 2) registers and the autotuner picks.  Measured on
+// 2^20 events, ms at 168 / 128 / 85: gg>ggg 4.22 / 5.25 / 6.95, gg>gg 0.91 /
+// 0.76 / 0.66, uu~>gg 0.68 / 0.76 / 0.60.  The FP64 bodies come at 128.  A
+// module that also held uncapped FP32 variants measured 25-45 % slower on the
+// same 128-register kernel, so none is built.
 template <typename R, typename Body, int MINB, int MAXT>
 __global__ void __launch_bounds__(MAXT, MINB) gen_kernel(const DevProgram P, const AmpLaunch A,
                                                                    const AmpConfig C) {
