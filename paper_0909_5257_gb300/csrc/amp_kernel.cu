@@ -493,12 +493,47 @@ static int gen_body_variant(const DevProgram& p, int cap) {
   return 2 * cap + (p.family == FAM_TWO_LINES && p.n_ext == 5 && cap == 1 ? 1 : 0);
 }
 
+int sm_count() {
+  static int n = 0;
+  if (n == 0) {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    n = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0 ? v : 1;
+  }
+  return n;
+}
+
+size_t gen_smem(const DevProgram& p, int E, int threads, size_t real) {
+  return (((size_t)E * event_table_stride(p.n_ext, p.n_masks) * real + 7) & ~size_t(7)) + (size_t)threads * 16 + 16;
+}
+
+// Fewer events than one plan tile per SM: a share of them for every SM instead of
+// full tiles on a few.  Preparation and the per-event finish, serial chains over
+// the tile's items, get shorter, and so does the whole call; the threads cover
+// the items of a preparation pass (legs, masks and check) as well as the lanes.
+// Never more than one CTA per SM: two small ones each fetch the long
+// straight-line code for themselves (uu~>ggg, 777 events: 33 us on 259 CTAs).
+// Measured, one call of 777 events (mixed, plan tiles -> spread): uu~>ggg 24.3
+// -> 20.9 us, gg>gg 23.1 -> 15.5, uu~>gg 18.8 -> 15.0, gg>ggg 35.5 -> 31.2,
+// uu>uug 21.9 -> 18.7; gg>gg in FP64 54.0 -> 41.6.
+AmpConfig gen_spread(const DevProgram& p, const AmpConfig& plan, int64_t n_events, size_t real) {
+  const int64_t sms = sm_count();
+  const int E = (int)std::max<int64_t>(1, (n_events + sms - 1) / sms);
+  if (E >= plan.E_cta) return plan;
+  AmpConfig c = plan;
+  c.E_cta = E;
+  const int items = std::max({c.H, (int)p.n_ext, (int)p.n_masks + 1});
+  c.threads = std::min(plan.threads, (E * items + 31) / 32 * 32);
+  c.smem = gen_smem(p, E, c.threads, real);
+  c.grid = (int)((n_events + E - 1) / E);
+  return c;
+}
+
 static AmpConfig plan_generated(const DevProgram& p, bool fp64, int H, int64_t n_events, int num_sms) {
   AmpConfig best;
   best.H = H;
   best.jamp_in_smem = true;
   best.slots_in_smem = true;
-  const int tab_stride = event_table_stride(p.n_ext, p.n_masks);
   double best_score = -1;
   // default: the 128-register variant (mea_autotune also tries 85 and 168 registers)
   const int regvar = fp64 ? 0 : (p.gen_forced >= 0 ? p.gen_forced : gen_body_variant(p, 0));
@@ -509,7 +544,7 @@ static AmpConfig plan_generated(const DevProgram& p, bool fp64, int H, int64_t n
   for (int E = 1; E * H <= max_threads; ++E) {
     int threads = ((E * H + 31) / 32) * 32;
     if (threads > max_threads) break;
-    size_t sm = (((size_t)E * tab_stride * (fp64 ? 8 : 4) + 7) & ~size_t(7)) + (size_t)threads * 16 + 16;
+    size_t sm = gen_smem(p, E, threads, fp64 ? 8 : 4);
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, sm) != cudaSuccess) per_sm = 0;
     if (per_sm < 1) continue;  // this tile cannot be resident: skip it
@@ -528,7 +563,7 @@ static AmpConfig plan_generated(const DevProgram& p, bool fp64, int H, int64_t n
   if (best_score < 0) {  // nothing resident at all: one warp per tile
     best.E_cta = std::max(1, 32 / std::max(H, 1));
     best.threads = ((best.E_cta * H + 31) / 32) * 32;
-    best.smem = (((size_t)best.E_cta * tab_stride * (fp64 ? 8 : 4) + 7) & ~size_t(7)) + (size_t)best.threads * 16 + 16;
+    best.smem = gen_smem(p, best.E_cta, best.threads, fp64 ? 8 : 4);
     best.grid = num_sms;
     best.regvar = regvar;
   }

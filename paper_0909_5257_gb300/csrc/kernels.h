@@ -148,6 +148,11 @@ struct AmpConfig {
 // global memory, both of which live in L1.
 int carveout_percent(const AmpConfig& c);
 
+int sm_count();  // of the current device
+
+// The straight-line kernels' tile for a call of n_events (dynamic shared memory for a real of that many bytes).
+AmpConfig gen_spread(const DevProgram& p, const AmpConfig& plan, int64_t n_events, size_t real);
+
 // Choose tile shape and grid for a program, precision and helicity mode.
 AmpConfig plan_amp(const DevProgram& p, bool fp64, int H, int64_t n_events, int num_sms,
                    size_t max_smem_per_block, size_t smem_per_sm, int events_per_tile_hint = 0);

@@ -117,16 +117,6 @@ __global__ void __launch_bounds__(kOrdThreads) ordered_kernel(const DevProgram P
   }
 }
 
-int sm_count() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    n = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0 ? v : 1;
-  }
-  return n;
-}
-
 }  // namespace
 
 bool ordered_supported(const DevProgram& p, bool fp64, int H) { return fp64 && p.ord_stages != nullptr && H == p.ord_lanes; }
