@@ -43,14 +43,24 @@ namespace {
 
 using namespace tc;
 
-constexpr int kThreads = 256;  // 8 warps convert; warps w and w+4 share TMEM lanes 32(w%4).. in the epilogue
 constexpr int kM = 128;        // tile rows (64 pairs x {re, im})
 constexpr int kKC = 64;        // K elements per stage
 constexpr int kPlaneA = kM * kKC * 2;
 
 __host__ __device__ constexpr size_t stage_bytes(int nc) { return (size_t)3 * kPlaneA + (size_t)2 * nc * kKC * 2; }
 
-__global__ void __launch_bounds__(kThreads, 1) colour_gemm_kernel(ColourGemmArgs g) {
+// kParts threads work on a row: they convert its operand digits between them and
+// warps w, w + 4, .. share TMEM lanes 32 (w % 4).. in the epilogue.  Latency of the
+// conversion and the epilogue bounds the kernel (few warps per scheduler, the
+// tensor core mostly waits), so four where shared memory holds one CTA per SM:
+// 16 warps instead of 8.  Two where it holds two (nc = 32), which have 16 warps
+// between them already: four leave registers for one CTA only.  Measured,
+// us/event, two -> four: gg>5g 0.613 -> 0.452, uu>uu+3g 0.224 -> 0.179, uu~>5g
+// 0.0957 -> 0.0865, gg>4g 0.020 both; uu~>4g (nc = 32) 0.0146 -> 0.0169.
+template <int kParts>
+__global__ void __launch_bounds__(kParts * kM, 1) colour_gemm_kernel(ColourGemmArgs g) {
+  constexpr int kThreads = kParts * kM;
+  constexpr int kGroups = kKC / 8 / kParts;  // groups of 8 K elements per thread and stage
   extern __shared__ __align__(1024) unsigned char smem[];
   const int t = threadIdx.x;
   const int warp = t >> 5;
@@ -62,9 +72,9 @@ __global__ void __launch_bounds__(kThreads, 1) colour_gemm_kernel(ColourGemmArgs
   int* abort_flag = reinterpret_cast<int*>(tslot + 1);
   float* rscale = reinterpret_cast<float*>(tslot + 4);           // [128] per-row scale 2^-e
   // scratch that lives in stage 1's first operand plane while no MMA reads it:
-  // row-maximum halves at the start of a tile, per-(row, half) values at its end
-  float* rmax = reinterpret_cast<float*>(smem + SB);                     // [256]
-  double* part = reinterpret_cast<double*>(smem + SB + kThreads * 4);    // [256]
+  // row-maximum parts at the start of a tile, per-(row, part) values at its end
+  float* rmax = reinterpret_cast<float*>(smem + SB);                     // [kThreads]
+  double* part = reinterpret_cast<double*>(smem + SB + kThreads * 4);    // [kThreads]
 
   {
     // the layout above must fit the dynamic shared memory of this launch
@@ -102,7 +112,7 @@ __global__ void __launch_bounds__(kThreads, 1) colour_gemm_kernel(ColourGemmArgs
   const uint32_t idesc = make_idesc(kM, NC);
   const bool use_blo = g.b_lo != nullptr;
   const int row = t & (kM - 1);
-  const int half = t >> 7;  // conversion: k groups of this thread; epilogue: column half
+  const int sub = t >> 7;  // conversion: k groups of this thread; epilogue: blocks of 16 columns
 
   auto wait_buf = [&](int b) -> bool {
     if (!outstanding[b]) return true;
@@ -131,7 +141,7 @@ __global__ void __launch_bounds__(kThreads, 1) colour_gemm_kernel(ColourGemmArgs
     {
       float mx = 0.f;
       if (row_ok)
-        for (int k4 = half; 4 * k4 < m; k4 += 2) {
+        for (int k4 = sub; 4 * k4 < m; k4 += kParts) {
           const float4 v = jrow4[k4];
           const int k = 4 * k4;
           mx = fmaxf(mx, fabsf(v.x));
@@ -142,7 +152,9 @@ __global__ void __launch_bounds__(kThreads, 1) colour_gemm_kernel(ColourGemmArgs
       rmax[t] = mx;
       __syncthreads();
       if (t < kM) {
-        mx = fmaxf(rmax[t], rmax[t + kM]);
+        mx = rmax[t];
+#pragma unroll
+        for (int k = 1; k < kParts; ++k) mx = fmaxf(mx, rmax[t + k * kM]);
         int e = 0;
         if (mx > 0.f && isfinite(mx)) frexpf(mx, &e);
         rscale[t] = ldexpf(1.f, max(-120, min(120, 14 - e)));
@@ -150,14 +162,14 @@ __global__ void __launch_bounds__(kThreads, 1) colour_gemm_kernel(ColourGemmArgs
       __syncthreads();
     }
     const float sc = rscale[row];
-    float acc_hi = 0.f, acc_lo = 0.f;  // Dot2 of this thread's (row, column half)
-    float pj[4][8];                    // prefetched J chunk: 4 groups of 8 columns
+    float acc_hi = 0.f, acc_lo = 0.f;  // Dot2 of this thread's (row, columns)
+    float pj[kGroups][8];              // prefetched J chunk: groups of 8 columns
 
     auto prefetch = [&](int it) {
       const int kc = it % n_kc;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int kk0 = kc * kKC + (half + 2 * j) * 8;
+      for (int j = 0; j < kGroups; ++j) {
+        const int kk0 = kc * kKC + (sub + kParts * j) * 8;
         float4 v0 = make_float4(0.f, 0.f, 0.f, 0.f), v1 = v0;
         if (row_ok && kk0 < m) {
           v0 = jrow4[kk0 / 4];
@@ -182,7 +194,7 @@ __global__ void __launch_bounds__(kThreads, 1) colour_gemm_kernel(ColourGemmArgs
       bulk_g2s(b_hi, g.b_hi + tile_off, bytes, &kbar[st]);
       if (use_blo) bulk_g2s(b_lo, g.b_lo + tile_off, bytes, &kbar[st]);
     };
-    // epilogue of iteration it (buffer it % 2): this thread's row, its half of the columns
+    // epilogue of iteration it (buffer it % 2): this thread's row, its blocks of 16 columns
     auto epilogue = [&](int it) {
       const int b = it & 1;
       if (!wait_buf(b)) return;
@@ -190,7 +202,7 @@ __global__ void __launch_bounds__(kThreads, 1) colour_gemm_kernel(ColourGemmArgs
       const int n0 = (it / n_kc) * NC;
       const uint32_t lane = (uint32_t)((warp & 3) * 32) << 16;
       const uint32_t base = tmem + (uint32_t)(b * NC) + lane;
-      for (int c0 = half * (NC / 2); c0 < (half + 1) * (NC / 2); c0 += 16) {
+      for (int c0 = 16 * sub; c0 < NC; c0 += 16 * kParts) {
         float jvals[16];
         {
           float4 v[4] = {};
@@ -242,8 +254,8 @@ __global__ void __launch_bounds__(kThreads, 1) colour_gemm_kernel(ColourGemmArgs
       // J digits into this stage (free: its MMAs, iteration it-2, were waited
       // for by the epilogue of it-2 during iteration it-1)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int kg = half + 2 * j;
+      for (int j = 0; j < kGroups; ++j) {
+        const int kg = sub + kParts * j;
         __align__(16) __half hv[8], mv[8], lv[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
@@ -312,7 +324,12 @@ __global__ void __launch_bounds__(kThreads, 1) colour_gemm_kernel(ColourGemmArgs
     if (t < kM / 2) {
       const int64_t p = tile * (kM / 2) + t;
       const int a = 2 * t, b = 2 * t + 1;
-      if (p < g.n_pairs) g.pairval[p] = (part[a] + part[a + kM] + part[b] + part[b + kM]) * g.inv_den;
+      if (p < g.n_pairs) {
+        double v = 0.0;
+#pragma unroll
+        for (int k = 0; k < kParts; ++k) v += part[a + k * kM] + part[b + k * kM];
+        g.pairval[p] = v * g.inv_den;
+      }
     }
     __syncthreads();
   }
@@ -359,7 +376,7 @@ ColourTiles build_colour_tiles(const std::vector<int64_t>& K, int m) {
   ColourTiles T;
   T.m = m;
   const int nb = (m + 255) / 256;
-  T.nc = ((m + nb - 1) / nb + 31) / 32 * 32;  // column halves of the epilogue are multiples of 16
+  T.nc = ((m + nb - 1) / nb + 31) / 32 * 32;  // the epilogue works in blocks of 16 columns
   T.np = nb * T.nc;
   T.kp = ((m + kKC - 1) / kKC) * kKC;
   const int n_kc = T.kp / kKC;
@@ -392,14 +409,15 @@ cudaError_t launch_colour_gemm(const ColourGemmArgs& a, int num_sms, cudaStream_
   // the kernel reads J in 16-byte vectors within rows of ldj >= m entries
   if (a.ldj % 16 != 0 || a.m > a.ldj || (reinterpret_cast<uintptr_t>(a.J) & 15) != 0) return cudaErrorInvalidValue;
   size_t sm = colour_gemm_smem(a.nc);
-  cudaError_t e = ensure_dynamic_smem((const void*)colour_gemm_kernel, sm);
-  if (e != cudaSuccess) return e;
-  int64_t tiles = (2 * a.n_pairs + kM - 1) / kM;
   int tmem = 32;
   while (tmem < 2 * a.nc) tmem *= 2;
   const int per_sm = std::max(1, std::min<int>(512 / tmem, (int)((227u << 10) / sm)));
+  auto k = per_sm > 1 ? colour_gemm_kernel<2> : colour_gemm_kernel<4>;
+  cudaError_t e = ensure_dynamic_smem((const void*)k, sm);
+  if (e != cudaSuccess) return e;
+  int64_t tiles = (2 * a.n_pairs + kM - 1) / kM;
   int grid = (int)std::min<int64_t>(tiles, (int64_t)num_sms * per_sm);
-  colour_gemm_kernel<<<grid, kThreads, sm, s>>>(a);
+  k<<<grid, per_sm > 1 ? 2 * kM : 4 * kM, sm, s>>>(a);
   e = cudaGetLastError();
   if (e == cudaSuccess) ++launch_counter();
   return e;
