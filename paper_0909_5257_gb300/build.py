@@ -19,7 +19,7 @@ LIB = os.path.join(HERE, "libmea.so")
 BUILD_DIR = os.path.join(ROOT, "_build")
 SOURCES = ["generator.cpp", "helshare.cpp", "phased.cpp", "colour_base.cpp", "ordered.cpp", "amp_kernel.cu", "amp_hs_kernel.cu", "amp_phased_kernel.cu", "ordered_kernel.cu", "ps_kernel.cu", "api.cu", "colour_gemm.cu", "jamp_gemm.cu", "batch.cu",
            "server.cu", "peak.cu"]
-HEADERS = ["generator.h", "helshare.h", "phased.h", "colour_base.h", "ordered.h", "ordered_eval.cuh", "kernels.h", "colour_gemm.h", "jamp_gemm.h", "tc_common.cuh", "process.h", "heget.cuh", "amp_common.cuh", "gen_kernel.cuh", "codegen.cpp",
+HEADERS = ["generator.h", "helshare.h", "phased.h", "colour_base.h", "ordered.h", "ordered_eval.cuh", "kernels.h", "colour_gemm.h", "jamp_gemm.h", "tc_common.cuh", "process.h", "heget.cuh", "vertex_pinned.cuh", "amp_common.cuh", "gen_kernel.cuh", "codegen.cpp",
            "../phasespace/phasespace.h", "../../include/mea.h"]
 # Processes whose straight-line kernels are emitted at build time (live state
 # small enough for registers); every other process runs on the interpreter.

@@ -166,7 +166,7 @@ __device__ __forceinline__ cx<float> hs_amplitude(const Op& op, const X& x, cons
     }
     case OP_ADOT: {
       W4<float> w = x(0), p = x(1);
-      return part_contract<float>(w, p, (op.leg & 1u) != 0, (op.leg & 2u) != 0);
+      return part_contract<float>(w, p, (op.leg & 1u) != 0, false);  // sign: amp_negated
     }
     default:
       break;

@@ -107,7 +107,8 @@ __device__ __forceinline__ void st_slot(R* slots, int s, int L, int t, const W4<
 // `last`; fwd bit k (0..3) marks an input that is that output (read from the
 // register instead of the slot), bit 4 an output read by nothing but the next
 // op (kept in the register only, never stored).
-template <typename R, bool FWD = false>
+// AOUT: diagram amplitudes without the sign of OP_ADOT (amp_negated).
+template <typename R, bool FWD = false, bool AOUT = false>
 __device__ __forceinline__ bool eval_op(const Op& op, const DevProgram& P, R* slots, int L, int t, const R* et,
                                         const R* mt, uint32_t lam_bits, R g, R gg, cx<R>& amp,
                                         uint32_t fwd = 0u, W4<R>* last = nullptr) {
@@ -202,7 +203,7 @@ __device__ __forceinline__ bool eval_op(const Op& op, const DevProgram& P, R* sl
     case OP_ADOT: {  // diagram amplitude from its free wavefunction and the group's partial
       W4<R> w = in_(0);
       W4<R> p = in_(1);
-      amp = part_contract<R>(w, p, (op.leg & 1u) != 0, (op.leg & 2u) != 0);
+      amp = part_contract<R>(w, p, (op.leg & 1u) != 0, !AOUT && (op.leg & 2u) != 0);
       return true;
     }
     case OP_PVVV: {
@@ -356,9 +357,9 @@ __global__ void __launch_bounds__(kMaxThreads) amp_kernel(const DevProgram P, co
         cx<R> amp;
         bool is_amp;
         if constexpr (FWD) {
-          is_amp = eval_op<R, true>(w.op, P, slots, L, t, et, mt, lam_bits, g, gg, amp, __ldg(P.fwd + i), &last);
+          is_amp = eval_op<R, true, true>(w.op, P, slots, L, t, et, mt, lam_bits, g, gg, amp, __ldg(P.fwd + i), &last);
         } else {
-          is_amp = eval_op<R>(w.op, P, slots, L, t, et, mt, lam_bits, g, gg, amp);
+          is_amp = eval_op<R, false, AOUT>(w.op, P, slots, L, t, et, mt, lam_bits, g, gg, amp);
         }
         if (is_amp) take_amp(w.op.col_begin, w.op.col_count, amp);
       }

@@ -643,7 +643,7 @@ mea_status mea_create_process(const int* pdg, int n_ext, const mea_options* opts
     const int* de = nullptr;
     if ((e = upload(P, P->ph.rec, &dr)) != cudaSuccess || (e = upload(P, P->ph.units, &du)) != cudaSuccess ||
         (e = upload(P, P->ph.sets, &ds)) != cudaSuccess || (e = upload(P, P->ph.hv, &dv)) != cudaSuccess ||
-        (e = upload(P, P->ph.phase_end, &de)) != cudaSuccess) {
+        (e = upload(P, P->ph.list_end, &de)) != cudaSuccess) {
       destroy(P);
       return fail(MEA_E_CUDA, std::string("mea_create_process: ") + cudaGetErrorString(e));
     }
@@ -652,7 +652,7 @@ mea_status mea_create_process(const int* pdg, int n_ext, const mea_options* opts
     D.ph_sets = ds;
     D.ph_hv = dv;
     D.ph_end = de;
-    D.ph_phases = (int)P->ph.phase_end.size();
+    D.ph_phases = P->ph.phases;
     D.ph_area = P->ph.area;
     D.ph_H = P->ph.H;
     P->ph = mea::PhProgram();

@@ -46,6 +46,11 @@ enum OpType : uint8_t {
 
 // Amplitude operations (one per Feynman diagram, in diagram-ordinal order).
 inline bool is_amp_op(int t) { return t == OP_AVVV || t == OP_AGGGG || t == OP_AIOV || t == OP_ADOT; }
+// A contraction with the sign -1 (OP_ADOT's leg bit 1).  The kernels that write
+// every diagram amplitude out leave the sign away, and the coefficients of the
+// colour-amplitude stage (JampMap) carry it: the same sums, two operations per
+// amplitude less.
+inline bool amp_negated_bits(int t, int leg) { return t == OP_ADOT && (leg & 2) != 0; }
 // Vertex partials: like currents they fill a wavefunction slot.
 inline bool is_partial_op(int t) { return t >= OP_PVVV && t <= OP_PIOV; }
 
@@ -62,6 +67,7 @@ struct Op {
   uint32_t col_count;  // amplitudes: number of colour entries
 };
 static_assert(sizeof(Op) == 32, "Op must stay 32 bytes");
+inline bool amp_negated(const Op& op) { return amp_negated_bits(op.type, op.leg); }
 
 // One colour coefficient: J[alpha] += (re + i im) * amplitude.
 struct ColEntry {

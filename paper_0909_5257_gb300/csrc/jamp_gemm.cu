@@ -486,7 +486,7 @@ JampMap build_jamp_map(const Program& p) {
     if (!is_amp_op(op.type)) continue;
     for (uint32_t k = 0; k < op.col_count; ++k) {
       const ColEntry& c = p.col[op.col_begin + k];
-      const int n = c.re / g;
+      const int n = (amp_negated(op) ? -c.re : c.re) / g;
       colw[c.alpha] += std::abs(n);
       M.weight[d] += (float)std::abs((int)c.re);
       C[(size_t)c.alpha * kd + d] += n;

@@ -69,7 +69,7 @@ struct DevProgram {
   int hsp_area = 0;                     // prologue variants per event
   bool hsp_only = false;                // amplitude-output mode: plan and tune the split kernel only
   // phased evaluation (phased.h), or null: units, their records, the end of
-  // each phase, leg-set tables and the variant of every leg set per combination
+  // each phase's lists, leg-set tables and the variant of every leg set per combination
   const PhUnit* ph_units = nullptr;
   const uint32_t* ph_rec = nullptr;
   const int* ph_end = nullptr;

@@ -98,8 +98,8 @@ PhProgram build_phased(const Program& P, const HelLanes& lanes, const std::vecto
       holder.at(op.out) = i;
     }
   }
-  check(n_amp < 0x7FFF && weight.size() == (size_t)n_amp && row.size() == weight.size(),
-        "diagram ordinals of 15 bits");
+  check(n_amp < 0x10000 && weight.size() == (size_t)n_amp && row.size() == weight.size(),
+        "diagram ordinals of 16 bits");
 
   // fused: read once, by a contraction, with n - 2 legs and at least two rounds
   std::vector<char> fused(n_ops, 0), stored(n_ops, 0);
@@ -284,16 +284,16 @@ PhProgram build_phased(const Program& P, const HelLanes& lanes, const std::vecto
             c.u.sp = (uint8_t)(all & ~g.first.sf);
             c.u.np = (uint8_t)np;
             PhOuterHead hd{};
-            for (int k = 0; k < np; ++k) hd.p[k] = (uint16_t)off[s.second[p0 + k]];
+            for (int k = 0; k < 4; ++k) hd.p[k] = 32u * (uint32_t)off[s.second[p0 + std::min(k, np - 1)]];
             put(&hd, sizeof hd);
             for (int q = 0; q < nf; ++q) {
               const int f = s.first[f0 + q];
               PhOuterRec r{};
-              r.f = (uint16_t)off[f];
+              r.f = 32u * (uint32_t)off[f];
               for (int k = 0; k < 4; ++k) r.d[k] = kPhNone;
               for (int k = 0; k < np; ++k) {
                 const int a = g.second[s.second[p0 + k]][f];
-                r.d[k] = (uint16_t)(row[ordinal[a]] | ((P.ops[a].leg & 2u) ? 0x8000 : 0));
+                r.d[k] = (uint32_t)row[ordinal[a]];
                 r.w[k] = weight[ordinal[a]];
               }
               put(&r, sizeof r);
@@ -316,6 +316,7 @@ PhProgram build_phased(const Program& P, const HelLanes& lanes, const std::vecto
       if (fused_amp[i] < 0) continue;
       const int t = fused_amp[i], p = src[4 * (size_t)i + 1];
       check((legs[t] & legs[p]) == 0, "fused current and partial share legs");
+      check((P.ops[i].leg & 1u) == ((P.ops[t].type == OP_FVI || P.ops[t].type == OP_FVO) ? 1u : 0u), "contraction of a fused current");
       int ph = block[p] >= 0 ? first_use + block[p] : -1;
       const int n_in = P.ops[t].n_in;
       for (int k = 0; k < n_in; ++k) {
@@ -326,6 +327,9 @@ PhProgram build_phased(const Program& P, const HelLanes& lanes, const std::vecto
       groups[{ph, legs[t], (int)P.ops[t].type}].push_back(i);
     }
     for (auto& g : groups) {
+      // currents with the same partial follow each other
+      std::stable_sort(g.second.begin(), g.second.end(),
+                       [&](int x, int y) { return src[4 * (size_t)x + 1] < src[4 * (size_t)y + 1]; });
       const uint32_t S = std::get<1>(g.first), SP = all & ~S;
       const std::vector<char> u = used(S);
       std::vector<int> vs;
@@ -338,7 +342,7 @@ PhProgram build_phased(const Program& P, const HelLanes& lanes, const std::vecto
         PhSet T;
         std::memset(&T, 0, sizeof T);
         for (auto& r : T.uh)
-          for (uint16_t& x : r) x = kPhNone;
+          for (uint16_t& x : r) x = kPhNoPair;
         std::vector<int> legs_of;
         for (int l = 0; l < n; ++l)
           if (S >> l & 1u) legs_of.push_back(l);
@@ -347,7 +351,7 @@ PhProgram build_phased(const Program& P, const HelLanes& lanes, const std::vecto
           const bool on = i < (int)vs.size();
           const int v = on ? vs[i] : vs[0];
           T.v[lane] = (uint8_t)v;
-          for (uint32_t m = 0; m < 32; ++m) T.sub[m][lane] = (uint8_t)pext8((uint32_t)v, m);
+          for (uint32_t m = 0; m < 32; ++m) T.sub[m][lane] = (uint16_t)(32u * pext8((uint32_t)v, m));
           int r = 0;
           for (int h = 0; h < H && on; ++h)
             if ((int)pext8(hbits[h], S) == v) {
@@ -358,6 +362,9 @@ PhProgram build_phased(const Program& P, const HelLanes& lanes, const std::vecto
         set_index[S] = (int)Q.sets.size();
         Q.sets.push_back(T);
       }
+      int rounds = 0;
+      for (int lane = 0; lane < 32; ++lane)
+        while (rounds < kPhRounds && Q.sets[set_index[S]].uh[rounds][lane] != kPhNoPair) ++rounds;
       const int per_pass = 32 >> lg;
       const size_t most = (size_t)std::max(8, 4 * per_pass);
       for (size_t b = 0; b < g.second.size(); b += most) {
@@ -369,24 +376,24 @@ PhProgram build_phased(const Program& P, const HelLanes& lanes, const std::vecto
         c.u.rec = here();
         c.u.set = (uint16_t)set_index[S];
         c.u.lanes = (uint8_t)lg;
+        c.u.rounds = (uint8_t)rounds;
         for (size_t q = 0; q < k; ++q) {
-          const int a = g.second[b + q], t = fused_amp[a], p = src[4 * (size_t)a + 1];
+          const int a = g.second[b + q], t = fused_amp[a];
           const Op& op = P.ops[t];
           PhFusedRec r{};
           for (int j = 0; j < op.n_in; ++j) {
             const int s = src[4 * (size_t)t + j];
-            r.in[j] = (uint16_t)off[s];
-            r.m[j] = (uint8_t)pext8(legs[s], S);
+            r.in[j] = 32u * (uint32_t)off[s];
+            r.m[j] = 64u * pext8(legs[s], S);
           }
-          r.plain = (uint8_t)(P.ops[a].leg & 1u);
-          if (op.type == OP_JVV) { r.r[0] = (uint8_t)op.min[0]; r.r[1] = (uint8_t)op.min[1]; }
-          r.r[2] = (uint8_t)op.mout;
-          r.p = (uint16_t)off[p];
-          r.d = (uint16_t)(row[ordinal[a]] | ((P.ops[a].leg & 2u) ? 0x8000 : 0));
+          if (op.type == OP_JVV) { r.r[0] = 32u * op.min[0]; r.r[1] = 32u * op.min[1]; }
+          r.r[2] = 32u * op.mout;
+          r.p = 32u * (uint32_t)off[src[4 * (size_t)a + 1]];
+          r.d = (uint32_t)row[ordinal[a]];
           r.w = weight[ordinal[a]];
           put(&r, sizeof r);
         }
-        c.cost = 80 + 280.0 * (double)((k + per_pass - 1) / per_pass);
+        c.cost = 150 + (120.0 + 40.0 * rounds) * (double)((k + per_pass - 1) / per_pass);
         c.phase = std::get<0>(g.first);
         units.push_back(c);
       }
@@ -449,14 +456,24 @@ PhProgram build_phased(const Program& P, const HelLanes& lanes, const std::vecto
       c.phase = best;
       load[best] += c.cost;
     }
-  // within a phase the costly units first: warp w takes units w, w + W, ...
+  // each phase's units onto kPhWarps lists, the costly ones first, each to the
+  // list with the least work; the warps of a CTA take lists w, w + W, ...
   std::stable_sort(units.begin(), units.end(), [](const Costed& a, const Costed& b) {
     return a.phase != b.phase ? a.phase < b.phase : a.cost > b.cost;
   });
-  for (auto& c : units) Q.units.push_back(c.u);
+  Q.phases = n_phases;
   for (int p = 0, i = 0; p < n_phases; ++p) {
-    while (i < (int)units.size() && units[i].phase == p) ++i;
-    Q.phase_end.push_back(i);
+    std::vector<std::vector<PhUnit>> list(kPhWarps);
+    std::vector<double> work(kPhWarps, 0.0);
+    for (; i < (int)units.size() && units[i].phase == p; ++i) {
+      const int l = (int)(std::min_element(work.begin(), work.end()) - work.begin());
+      list[l].push_back(units[i].u);
+      work[l] += units[i].cost;
+    }
+    for (auto& l : list) {
+      Q.units.insert(Q.units.end(), l.begin(), l.end());
+      Q.list_end.push_back((int)Q.units.size());
+    }
   }
   return Q;
 }

@@ -17,7 +17,7 @@
 //            four vertex partials over complementary leg sets, a lane per
 //            helicity combination, the partials held in registers;
 //   FUSED    currents of n_ext - 2 legs, a lane per variant, each contracted
-//            with the variants of its partial (a round per partial variant);
+//            with the variants of its partial (a round per variant);
 //   GENERIC  the remaining diagram amplitudes, a lane per combination.
 // The operations and their inputs are the per-lane program's (heget.cuh), so
 // the diagram amplitudes are the same bit for bit.
@@ -33,7 +33,7 @@ enum PhType : uint8_t { PH_PRODUCE = 0, PH_OUTER = 1, PH_FUSED = 2, PH_GENERIC =
 constexpr int kPhFree = 24;     // free wavefunctions per OUTER unit
 constexpr int kPhPartials = 4;  // partials per OUTER unit
 constexpr int kPhRounds = 4;    // variants of a two-leg partial
-constexpr int kPhMassSlots = 24;  // accumulators of the cancellation mass; the warps of a CTA divide it
+constexpr int kPhWarps = 12;    // unit lists per phase; the warps of a CTA divide it
 
 struct PhUnit {
   uint8_t type;   // PhType
@@ -45,7 +45,7 @@ struct PhUnit {
   uint8_t np;      // OUTER: partials
   uint16_t set;    // FUSED: leg-set table
   uint8_t lanes;   // FUSED: log2 of the lanes per current
-  uint8_t pad;
+  uint8_t rounds;  // FUSED: rounds in which some lane has a combination
 };
 static_assert(sizeof(PhUnit) == 16, "PhUnit must stay 16 bytes");
 
@@ -58,32 +58,32 @@ struct PhItem {
 };
 static_assert(sizeof(PhItem) == 16, "PhItem must stay 16 bytes");
 
-// OUTER: one header of four partial offsets, then per free wavefunction its
-// offset, the four diagrams (bit 15: negated; kPhNone: absent) and weights.
-constexpr uint16_t kPhNone = 0xFFFFu;
+// The records of the inner loops hold 32-bit words that are used as they are:
+// byte offsets into the area (variants of 32 bytes), into the event table's
+// rows (32 bytes each), rows of the amplitude buffer.
+
+// OUTER: one header of four partial blocks, then per free wavefunction its
+// block, and per partial the amplitude's row (kPhNone: absent) and weight.
+constexpr uint32_t kPhNone = 0xFFFFFFFFu;
 struct PhOuterHead {
-  uint16_t p[4];
-  uint32_t pad[2];
+  uint32_t p[4];
 };
 struct PhOuterRec {
-  uint16_t f, pad;
-  uint16_t d[4];
-  uint32_t pad2;
+  uint32_t f, pad[3];
+  uint32_t d[4];
   float w[4];
 };
-static_assert(sizeof(PhOuterHead) == 16 && sizeof(PhOuterRec) == 32, "OUTER records");
+static_assert(sizeof(PhOuterHead) == 16 && sizeof(PhOuterRec) == 48, "OUTER records");
 
-// FUSED: the current's input blocks (offset, legs within the set's table), its
-// rows, the partial's block, the diagram (bit 15: negated) and its weight.
+// FUSED: per current its input blocks, the inputs' legs (byte offset into
+// PhSet::sub), its rows, the partial's block, the amplitude's row and weight.
 struct PhFusedRec {
-  uint16_t in[3];
-  uint8_t m[3], plain;
-  uint8_t r[3], pad;
-  uint16_t p, d;
+  uint32_t in[3], d;
+  uint32_t m[3];
   float w;
-  uint32_t pad2[2];
+  uint32_t r[3], p;
 };
-static_assert(sizeof(PhFusedRec) == 32, "FUSED record");
+static_assert(sizeof(PhFusedRec) == 48, "FUSED record");
 
 struct PhGenericRec {
   uint8_t type, flags;  // flags: ADOT's leg bits
@@ -98,16 +98,18 @@ static_assert(sizeof(PhGenericRec) == 32, "GENERIC record");
 
 // FUSED: a leg set's variants that occur in the sum and, per round, the
 // partial's variant (low byte) and combination (high byte) of each.
+constexpr uint16_t kPhNoPair = 0xFFFFu;
 struct PhSet {
   uint8_t v[32];                    // variant of lane i
-  uint16_t uh[kPhRounds][32];       // kPhNone: none
-  uint8_t sub[32][32];              // [input legs, as bits of the set's legs][lane]: the input's variant
+  uint16_t uh[kPhRounds][32];       // kPhNoPair: none
+  uint16_t sub[32][32];             // [input legs, as bits of the set's legs][lane]: the input's variant x 32
 };
 
 struct PhProgram {
   std::vector<uint32_t> rec;       // records (16-byte words as 4 x uint32)
   std::vector<PhUnit> units;
-  std::vector<int> phase_end;      // end of each phase's units
+  std::vector<int> list_end;       // [phases][kPhWarps]: end of each list's units
+  int phases = 0;
   std::vector<PhSet> sets;
   std::vector<uint8_t> hv;         // [2^n_ext][128]: variant of the legs for combination h
   int area = 0;                    // variants per event

@@ -78,6 +78,9 @@ int main(int argc, char** argv) {
     if (P.n_diagrams % 5 == 0)
       for (int d = 0; d < P.n_diagrams; ++d) row[d] = P.n_diagrams - 1 - d;
     for (int d = 0; d < P.n_diagrams; ++d) row_of[row[d]] = d;
+    std::vector<char> negated;
+    for (const Op& op : P.ops)
+      if (is_amp_op(op.type)) negated.push_back(amp_negated(op));
     const PhProgram Q = build_phased(P, lanes, weight, row, 6800);
 
     std::mt19937_64 rng(0x5eed + a);
@@ -124,7 +127,7 @@ int main(int argc, char** argv) {
     std::vector<V> area(Q.area);
     std::vector<char> have(Q.area, 0);
     size_t i = 0;
-    for (size_t ph = 0; ph < Q.phase_end.size(); ++ph) {
+    for (int ph = 0; ph < Q.phases; ++ph) {
       std::set<int> rd, wr;
       auto ld = [&](uint32_t k) -> V {
         if (k >= (uint32_t)Q.area || !have[k]) { fault("read outside the area or before it is written"); return area[0]; }
@@ -133,15 +136,15 @@ int main(int argc, char** argv) {
       };
       std::vector<std::pair<int, V>> made_here;
       auto take = [&](cx<double> z, uint32_t d, float w, uint32_t h) {
-        if ((d & 0x7fffu) >= (uint32_t)P.n_diagrams) { fault("row"); return; }
-        const uint32_t dd = (uint32_t)row_of[d & 0x7fffu];
+        if (d >= (uint32_t)P.n_diagrams) { fault("row"); return; }
+        const uint32_t dd = (uint32_t)row_of[d];
         if (dd >= (uint32_t)P.n_diagrams || h >= (uint32_t)H) { fault("diagram or combination"); return; }
         if (w != weight[dd]) fault("weight");
-        if (d & 0x8000u) z = -z;
+        if (negated[dd]) z = -z;  // the sign the coefficients carry
         got[(size_t)h * P.n_diagrams + dd] = z;
         ++written[(size_t)h * P.n_diagrams + dd];
       };
-      for (; i < (size_t)Q.phase_end[ph]; ++i) {
+      for (; i < (size_t)Q.list_end[ph * kPhWarps + kPhWarps - 1]; ++i) {
         const PhUnit& U = Q.units[i];
         auto rec = [&](size_t at, void* to, size_t bytes) {
           if (4 * (U.rec + at) + bytes / 4 > Q.rec.size()) { fault("record"); std::memset(to, 0, bytes); return; }
@@ -166,13 +169,14 @@ int main(int argc, char** argv) {
             const int per = 32 >> U.lanes;
             for (int t = lane >> U.lanes; t < U.n; t += per) {
               PhFusedRec c;
-              rec(2 * t, &c, sizeof c);
+              rec(3 * t, &c, sizeof c);
               V x[4];
-              for (int j = 0; j < (U.op == OP_JGGG ? 3 : 2); ++j) x[j] = ld(c.in[j] + T.sub[c.m[j]][lane]);
-              const V y = made(U.op, 0, x, mrow(c.r[0]), mrow(c.r[1]), mrow(c.r[2]), mrow(c.r[2]));
+              for (int j = 0; j < (U.op == OP_JGGG ? 3 : 2); ++j) x[j] = ld((c.in[j] + T.sub[c.m[j] / 64][lane]) / 32);
+              const V y = made(U.op, 0, x, mrow(c.r[0] / 32), mrow(c.r[1] / 32), mrow(c.r[2] / 32), mrow(c.r[2] / 32));
               for (int r = 0; r < kPhRounds; ++r)
-                if (T.uh[r][lane] != kPhNone)
-                  take(part_contract<double>(y, ld(c.p + (T.uh[r][lane] & 255)), c.plain != 0, false), c.d, c.w, T.uh[r][lane] >> 8);
+                if (T.uh[r][lane] != kPhNoPair)
+                  take(part_contract<double>(y, ld(c.p / 32 + (T.uh[r][lane] & 255)), U.op == OP_FVI || U.op == OP_FVO, false), c.d, c.w,
+                       T.uh[r][lane] >> 8);
             }
           } else {
             const int h = 32 * U.pass + lane;
@@ -182,9 +186,9 @@ int main(int argc, char** argv) {
               rec(0, &hd, sizeof hd);
               for (int k = 0; k < U.n; ++k) {
                 PhOuterRec c;
-                rec(1 + 2 * k, &c, sizeof c);
+                rec(1 + 3 * k, &c, sizeof c);
                 for (int q = 0; q < U.np; ++q)
-                  take(part_contract<double>(ld(c.f + Q.hv[128 * U.sf + h]), ld(hd.p[q] + Q.hv[128 * U.sp + h]), U.op != 0, false),
+                  take(part_contract<double>(ld(c.f / 32 + Q.hv[128 * U.sf + h]), ld(hd.p[q] / 32 + Q.hv[128 * U.sp + h]), U.op != 0, false),
                        c.d[q], c.w[q], h);
               }
             } else {
@@ -194,7 +198,7 @@ int main(int argc, char** argv) {
                 V x[4];
                 const int n_in = c.type == OP_AGGGG ? 4 : (c.type == OP_ADOT ? 2 : 3);
                 for (int j = 0; j < n_in; ++j) x[j] = ld(c.in[j] + Q.hv[128 * c.m[j] + h]);
-                take(closed(c.type, c.flags, x, mrow(c.r[0]), mrow(c.r[1]), mrow(c.r[2])), c.d, c.w, h);
+                take(closed(c.type, c.flags & 1, x, mrow(c.r[0]), mrow(c.r[1]), mrow(c.r[2])), c.d, c.w, h);
               }
             }
           }
