@@ -12,7 +12,10 @@
 namespace mea {
 namespace tc {
 
-constexpr uint32_t kSpinLimit = 1u << 26;  // bounded waits: ~seconds, then an error flag
+// Polls of a bounded wait before it gives up and an error flag is set: 2 s, a
+// try_wait that finds nothing taking 3.8 us (2^26 of them, which were the bound
+// once, are 254 s).  What is waited for inside a CTA takes microseconds.
+constexpr uint32_t kSpinLimit = 1u << 19;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
