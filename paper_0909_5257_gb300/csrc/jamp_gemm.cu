@@ -35,9 +35,16 @@
 // into two shared-memory stages, a seventeenth issues the MMAs and the bulk
 // copies of the coefficient tiles (four stages); they meet at mbarriers, never
 // at a CTA barrier inside the loop, and the loads run two chunks ahead across
-// tile boundaries.  Every wait is bounded; on expiry the kernel records an
-// error in *status, drains its copies and MMAs with one more bounded wait,
-// frees its tensor memory and returns.
+// tile boundaries.
+//
+// Every mbarrier wait is bounded.  A wait that expires records an error in
+// *status and sets a flag that ends the others' waits.  Barriers have no bound, so
+// nobody may leave one that others stand at: a wait's outcome is made uniform
+// over its warp, and after the waits of a tile all converters meet at one
+// barrier that also votes -- each reaches it once per tile, whatever its waits
+// gave, and they go on or leave together.  The issuing thread, on every path,
+// waits (with a bound) for the copies and MMAs it has issued before the CTA's
+// shared and tensor memory go away.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -87,6 +94,19 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   return r;
 }
 __device__ __forceinline__ void bar_converters() { asm volatile("bar.sync 1, %0;" ::"n"(kConvert) : "memory"); }
+// the same barrier; true where `ok` is on all of them
+__device__ __forceinline__ bool vote_converters(bool ok) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.and.pred q, 1, %2, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}\n"
+      : "=r"(r)
+      : "r"((uint32_t)ok), "n"(kConvert)
+      : "memory");
+  return r != 0;
+}
 
 __host__ __device__ constexpr size_t tail_bytes() {
   // 2 + 2 + kBStages + 1 barriers, TMEM slot and abort flag, [kM] row scales, [8][kM] partial sums of |J|
@@ -191,8 +211,8 @@ __global__ void __launch_bounds__(kThreads, 1) jamp_gemm_kernel(JampGemmArgs g) 
           const int st = (int)(i & 1u);
           // the digits of chunk i (then the MMAs of chunk i - 2 are done too:
           // the converters waited for them before they wrote)
-          ok = mbar_wait_abort(&full[st], (i >> 1) & 1u, abort_flag) &&
-               mbar_wait_abort(&bfull[i % kBStages], (i / kBStages) & 1u, abort_flag);
+          ok = mbar_wait_abort(&full[st], (i >> 1) & 1u, abort_flag, g.spin_limit) &&
+               mbar_wait_abort(&bfull[i % kBStages], (i / kBStages) & 1u, abort_flag, g.spin_limit);
           if (!ok) break;
           copy();  // chunk i + 2 into the coefficient stage chunk i - 2 read
           fence_after();
@@ -212,14 +232,13 @@ __global__ void __launch_bounds__(kThreads, 1) jamp_gemm_kernel(JampGemmArgs g) 
           if (kc == n_kc - 1) mma_commit(done);
         }
       }
-      if (!ok) {
-        expired();
-        // copies in flight land, and the MMAs issued finish, before the CTA's
-        // shared and tensor memory go away
-        for (uint32_t k = i; k < issued; ++k) mbar_wait(&bfull[k % kBStages], (k / kBStages) & 1u);
-        for (uint32_t k = i > 2 ? i - 2 : 0; k < i; ++k) mbar_wait(&empty[k & 1u], (k >> 1) & 1u);
-      }
+      if (!ok) expired();
+      // copies in flight land, and the MMAs issued finish, before the CTA's shared
+      // and tensor memory go away (also where only converters gave up)
+      for (uint32_t k = i; k < issued; ++k) mbar_wait(&bfull[k % kBStages], (k / kBStages) & 1u);
+      for (uint32_t k = i > 2 ? i - 2 : 0; k < i; ++k) mbar_wait(&empty[k & 1u], (k >> 1) & 1u);
     }
+    __syncwarp();
   } else {
     // ---- digits: thread -> (pair, 8 consecutive diagrams)
     const int p = t & (kPairs - 1), kg = t >> 6;
@@ -257,6 +276,12 @@ __global__ void __launch_bounds__(kThreads, 1) jamp_gemm_kernel(JampGemmArgs g) 
       const int64_t pair = (int64_t)tile * kPairs + p;
       return pair < g.n_pairs ? __ldg(reinterpret_cast<const float2*>(g.rowmax) + pair) : make_float2(0.f, 0.f);
     };
+    // a bounded wait with one outcome for the warp
+    auto wait = [&](uint64_t* bar, uint32_t phase) {
+      const bool got = mbar_wait_abort(bar, phase, abort_flag, g.spin_limit);
+      if (!got) expired();
+      return __all_sync(0xffffffffu, got) != 0;
+    };
     uint32_t i = 0, tile_no = 0;
     Walk ahead, w, w_next;
     ahead.start(ns, begin);
@@ -266,8 +291,7 @@ __global__ void __launch_bounds__(kThreads, 1) jamp_gemm_kernel(JampGemmArgs g) 
     ahead.next_chunk(ns, begin, d_tile, d_split);
     w.start(ns, begin);
     float2 mx = row_max(w.tile);
-    bool ok = true;
-    for (; w.tile < n_tiles && ok; w = w_next, ++tile_no) {
+    for (; w.tile < n_tiles; w = w_next, ++tile_no) {
       const float s_re = scale_of(mx.x), s_im = scale_of(mx.y);
       w_next = w;
       w_next.next_work(ns, begin, d_tile, d_split);
@@ -280,7 +304,7 @@ __global__ void __launch_bounds__(kThreads, 1) jamp_gemm_kernel(JampGemmArgs g) 
       const int n_kc = begin[w.split + 1] - begin[w.split];
       auto step = [&](ABuf& pa) {
         const int st = (int)(i & 1u);
-        if (i >= 2 && !mbar_wait_abort(&empty[st], ((i - 2) >> 1) & 1u, abort_flag)) return false;
+        if (i >= 2 && !wait(&empty[st], ((i - 2) >> 1) & 1u)) return false;
         unsigned char* a_h = smem + (size_t)st * 3 * kStageA;
         // x = a s, r1 = (x - h) w, r2 = (r1 - m) w: every product by the powers
         // of two s and w and every difference of a value and its nearest
@@ -329,6 +353,7 @@ __global__ void __launch_bounds__(kThreads, 1) jamp_gemm_kernel(JampGemmArgs g) 
         return true;
       };
       // the buffers alternate over all chunks of the CTA (i even: pa0)
+      bool ok = true;
       int kc = 0;
       if (i & 1u) {
         ok = step(pa1);
@@ -336,9 +361,8 @@ __global__ void __launch_bounds__(kThreads, 1) jamp_gemm_kernel(JampGemmArgs g) 
       }
       for (; ok && kc + 1 < n_kc; kc += 2) ok = step(pa0) && step(pa1);
       if (ok && kc < n_kc) ok = step(pa0);
-      if (!ok) break;
-      ok = mbar_wait_abort(done, tile_no & 1u, abort_flag);
-      if (!ok) break;
+      ok = ok && wait(done, tile_no & 1u);
+      if (!vote_converters(ok)) break;  // also: row scales written
       fence_after();
 
       // ---- epilogue: warp -> tensor-memory lanes 32 (warp mod 4) .., a quarter of the columns
@@ -348,7 +372,6 @@ __global__ void __launch_bounds__(kThreads, 1) jamp_gemm_kernel(JampGemmArgs g) 
       const uint32_t lane = (uint32_t)((warp & 3) * 32) << 16;
       const int lrow = (warp & 3) * 32 + (t & 31);
       const int quarter = warp >> 2;
-      bar_converters();  // row scales written
       if (n_kk == 0) {
         const int64_t pair = mt * kPairs + (lrow & (kPairs - 1));
         const float back = (float)g.cfac / rscale[lrow];  // cfac (1 or 2) times a power of two
@@ -451,7 +474,6 @@ __global__ void __launch_bounds__(kThreads, 1) jamp_gemm_kernel(JampGemmArgs g) 
       }
       bar_converters();  // row scales and sums free for the next tile
     }
-    if (!ok) expired();
   }
   fence_before();
   __syncthreads();
@@ -555,6 +577,7 @@ size_t jamp_gemm_smem(const JampGemmArgs& a) {
 }
 
 cudaError_t launch_jamp_gemm(const JampGemmArgs& a, int num_sms, cudaStream_t s) {
+  static_assert(JampGemmArgs().spin_limit == kSpinLimit, "the default of a launch");
   if (a.n_pairs <= 0) return cudaSuccess;
   if (a.n_pairs > (int64_t)1 << 36) return cudaErrorInvalidValue;  // tile numbers are 32-bit
   if (a.nc < 16 || a.nc > kMaxNC || a.nc % 16 != 0 || a.mb > a.m || a.mb > a.nc * a.n_splits) return cudaErrorInvalidValue;

@@ -75,8 +75,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t phase, uint32_
 }
 
 // The same, given up when *abort is set by another thread of the CTA.
-__device__ __forceinline__ bool mbar_wait_abort(uint64_t* bar, uint32_t phase, const volatile int* abort) {
-  for (uint32_t i = 0; i < kSpinLimit; ++i) {
+__device__ __forceinline__ bool mbar_wait_abort(uint64_t* bar, uint32_t phase, const volatile int* abort,
+                                                uint32_t limit = kSpinLimit) {
+  for (uint32_t i = 0; i < limit; ++i) {
     if (mbar_try_wait(bar, phase)) return true;
     if (*abort) return false;
   }

@@ -1,12 +1,22 @@
-// Bounded waits of the tensor-core GEMMs that run out: a wait with the usual
-// limit that nothing ends takes seconds.  Prints its time; exit status 1 on a fault.
+// Bounded waits of the tensor-core GEMMs that run out.  For every process given on
+// the command line the colour-amplitude GEMM runs on random diagram amplitudes with the usual limit, then with limits of 0 polls (every wait
+// expires at once), 1, 2, .. polls: each launch must end without an error, report
+// an expiry in its status word or none, and leave the next launch with the
+// usual limit to give the first one's results bit for bit.  Prints per process
+// the launches with an expiry; exit status 1 on a fault.
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
+#include <cstring>
+#include <random>
+#include <string>
 #include <vector>
 
 #include "colour_gemm.h"
+#include "generator.h"
+#include "jamp_gemm.h"
 #include "tc_common.cuh"
 
 using namespace mea;
@@ -30,7 +40,9 @@ static T* up(const std::vector<T>& v) {
   return static_cast<T*>(d);
 }
 
-int main() {
+int main(int argc, char** argv) {
+  int sms = 0;
+  ck(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0), "device");
   {
     // a wait with the usual limit that nothing ends: seconds
     std::vector<int> status(1, 0);
@@ -48,6 +60,103 @@ int main() {
     std::printf("bound %.0f ms\n", ms);
     need(status[0] == 1 && ms < 10000, "bound of a wait");
     cudaFree(s);
+  }
+  for (int arg = 1; arg < argc; ++arg) {
+    std::vector<int> pdg;
+    std::string s = argv[arg];
+    for (size_t p = 0; p < s.size();) {
+      size_t e = s.find(',', p);
+      if (e == std::string::npos) e = s.size();
+      pdg.push_back(std::atoi(s.substr(p, e - p).c_str()));
+      p = e + 1;
+    }
+    const Program P = build_program(pdg);
+    const JampMap M = build_jamp_map(P);
+    need(M.ok, "coefficients");
+    const int64_t n = 64 * 3 * (int64_t)sms + 37;  // several tiles per CTA, a ragged last one
+    const int64_t lda = (2 * n + 127) / 128 * 128;
+    const int ldj = (P.n_jamp + 15) / 16 * 16;
+    std::mt19937_64 rng(0x5eed + arg);
+    std::normal_distribution<float> gauss;
+    std::vector<float> A((size_t)M.kd * lda, 0.f), rowmax(2 * n, 0.f);
+    for (int d = 0; d < M.kd; ++d)
+      for (int64_t r = 0; r < 2 * n; ++r) {
+        const float v = gauss(rng);
+        A[(size_t)d * lda + r] = v;
+        rowmax[r] = std::max(rowmax[r], std::fabs(v));
+      }
+    std::vector<float> J((size_t)2 * n * ldj), jabs((size_t)M.n_splits * n);
+    std::vector<int> status(1, 0);
+    JampGemmArgs g;
+    g.A = up(A);
+    g.lda = lda;
+    g.rowmax = up(rowmax);
+    g.n_pairs = n;
+    g.kd = M.kd; g.m = M.m; g.mb = M.mb; g.nc = M.nc; g.n_splits = M.n_splits; g.q = M.q; g.cfac = M.cfac;
+    g.tiles = up(M.tiles);
+    g.chunks = up(M.chunks);
+    g.split_begin = up(M.split_begin);
+    g.n_chunks = (int)M.chunks.size();
+    g.kk_index = up(M.kk_index);
+    g.kk_term = up(M.kk_term);
+    g.kk_terms = (int)M.kk_term.size();
+    g.J = up(J);
+    g.ldj = ldj;
+    g.jabs = up(jabs);
+    g.status = up(status);
+    auto launched = [&](cudaError_t e) {  // its status word
+      ck(e, "launch");
+      ck(cudaDeviceSynchronize(), "kernel");
+      int v = 0;
+      ck(cudaMemcpy(&v, g.status, sizeof v, cudaMemcpyDeviceToHost), "status");
+      ck(cudaMemset(g.status, 0, sizeof v), "status");
+      return v;
+    };
+    // a diagram amplitude's share in colour amplitude alpha, for the reference
+    std::vector<std::vector<std::pair<int, double>>> row(P.n_jamp);
+    int d = 0;
+    for (const Op& op : P.ops) {
+      if (!is_amp_op(op.type)) continue;
+      for (uint32_t k = 0; k < op.col_count; ++k) {
+        const ColEntry& e = P.col[op.col_begin + k];
+        row[e.alpha].push_back({M.row[d], amp_negated(op) ? -(double)e.re : (double)e.re});
+      }
+      ++d;
+    }
+    std::vector<float> J0;
+    int expired = 0;
+    for (uint32_t polls : {kDefault, 0u, kDefault, 1u, 2u, 3u, 4u, 8u, 16u, 64u, 256u, kDefault}) {
+      g.spin_limit = polls;
+      const bool whole = polls == kDefault;
+      const int v = launched(launch_jamp_gemm(g, sms, nullptr));
+      need(whole ? v == 0 : (v == 0 || v == 1), "status of the colour-amplitude GEMM");
+      need(polls != 0 || v == 1, "no poll, no expiry (colour amplitudes)");
+      expired += v;
+      if (whole) {
+        ck(cudaMemcpy(J.data(), g.J, J.size() * 4, cudaMemcpyDeviceToHost), "J");
+        if (J0.empty()) {
+          J0 = J;
+          for (int64_t p : {(int64_t)0, (int64_t)63, n / 2, n - 1})
+            for (int ri = 0; ri < 2; ++ri)
+              for (int a = 0; a < P.n_jamp; ++a) {
+                double ref = 0, mag = 0;
+                for (auto& x : row[a]) {
+                  const double t = x.second * A[(size_t)x.first * lda + 2 * p + ri];
+                  ref += t;
+                  mag += std::fabs(t);
+                }
+                // FP32 result, digits cut 27 bits or more below the row's largest amplitude
+                need(std::fabs(J0[(size_t)(2 * p + ri) * ldj + a] - ref) <= 2e-7 * mag + 1e-7 * std::fabs(ref), "colour amplitude");
+              }
+        }
+        need(!std::memcmp(J.data(), J0.data(), J.size() * 4), "colour amplitudes after an expiry");
+      }
+    }
+    std::printf("%s %d\n", argv[arg], expired);
+    for (const void* q : {(const void*)g.A, (const void*)g.rowmax, (const void*)g.tiles, (const void*)g.chunks, (const void*)g.split_begin,
+                          (const void*)g.kk_index, (const void*)g.kk_term, (const void*)g.J, (const void*)g.jabs,
+                          (const void*)g.status})
+      cudaFree(const_cast<void*>(q));
   }
   return faults ? 1 : 0;
 }

@@ -1,5 +1,8 @@
-"""Waits of the tensor-core GEMMs that run out (tests/native/wait_expiry.cu): the
-usual limit is a matter of seconds."""
+"""Waits of the tensor-core colour-amplitude GEMM (jamp_gemm.cu) that run out: a
+launch whose waits expire, at once or somewhere on the way, ends by itself with
+its status word set and leaves the context usable
+(tests/native/wait_expiry.cu).  One column block with derived columns, one
+without, and two blocks."""
 import os
 import subprocess
 
@@ -18,5 +21,10 @@ def test_expired_waits_end_the_launch(tmp_path):
     subprocess.run([build.nvcc()] + build.ARCH + ["-O1", "-std=c++17", "-I", build.CSRC, "-o", exe,
                     os.path.join(HERE, "native", "wait_expiry.cu"), lib,
                     "-Xlinker", "-rpath=" + os.path.dirname(lib)], check=True)
-    r = subprocess.run([exe], capture_output=True, text=True, timeout=240)
+    procs = ["21,21,21,21,21,21", "2,-2,21,21,21,21", "2,2,2,2,21,21,21"]
+    r = subprocess.run([exe] + procs, capture_output=True, text=True, timeout=240)
     assert r.returncode == 0, r.stdout + r.stderr
+    rows = [line.split() for line in r.stdout.splitlines()[1:]]
+    assert [row[0] for row in rows] == procs
+    for name, expired in rows:
+        assert int(expired) >= 1, name
