@@ -87,7 +87,9 @@ __global__ void __launch_bounds__(kParts * kM, 1) colour_gemm_kernel(ColourGemmA
   }
   uint32_t tmem_cols = 32;
   while (tmem_cols < (uint32_t)(2 * NC)) tmem_cols <<= 1;
-  uint32_t kphase[2] = {0u, 0u};  // thread 0: next phase of each stage's K-tile barrier
+  // thread 0: next phase of each stage's K-tile barrier, and whether a copy that completes it is in flight
+  uint32_t kphase[2] = {0u, 0u};
+  bool kpending[2] = {false, false};
   if (t == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
@@ -114,14 +116,16 @@ __global__ void __launch_bounds__(kParts * kM, 1) colour_gemm_kernel(ColourGemmA
   const int row = t & (kM - 1);
   const int sub = t >> 7;  // conversion: k groups of this thread; epilogue: blocks of 16 columns
 
+  // one outcome for the warp: what follows a wait is executed by whole warps
+  // (tensor-memory loads), and lanes may see an expiry or the flag at different times
   auto wait_buf = [&](int b) -> bool {
     if (!outstanding[b]) return true;
-    if (*abort_flag) return false;
-    if (!mbar_wait(&bar[b], phase[b])) {
+    bool got = false;
+    if (!*abort_flag && !(got = mbar_wait(&bar[b], phase[b], g.spin_limit))) {
       atomicExch(abort_flag, 1);
       if (g.status) atomicExch(g.status, 1);
-      return false;  // left outstanding: drained once more before TMEM is freed
     }
+    if (!__all_sync(0xffffffffu, got)) return false;  // left outstanding: drained once more before TMEM is freed
     phase[b] ^= 1u;
     outstanding[b] = 0;
     return true;
@@ -191,6 +195,7 @@ __global__ void __launch_bounds__(kParts * kM, 1) colour_gemm_kernel(ColourGemmA
       const size_t tile_off = ((size_t)nb * n_kc + kc) * NC * kKC;
       const uint32_t bytes = (uint32_t)(NC * kKC * 2);
       mbar_expect_tx(&kbar[st], use_blo ? 2 * bytes : bytes);
+      kpending[st] = true;
       bulk_g2s(b_hi, g.b_hi + tile_off, bytes, &kbar[st]);
       if (use_blo) bulk_g2s(b_lo, g.b_lo + tile_off, bytes, &kbar[st]);
     };
@@ -278,13 +283,15 @@ __global__ void __launch_bounds__(kParts * kM, 1) colour_gemm_kernel(ColourGemmA
       fence_after();
       if (t == 0 && !*abort_flag) {
         // this stage's K tiles
-        if (!mbar_wait(&kbar[st], kphase[st])) {
+        if (mbar_wait(&kbar[st], kphase[st], g.spin_limit)) {
+          kphase[st] ^= 1u;
+          kpending[st] = false;
+        } else {
           atomicExch(abort_flag, 1);
           if (g.status) atomicExch(g.status, 1);
         }
-        kphase[st] ^= 1u;
       }
-      if (!*abort_flag) {
+      if (!__any_sync(0xffffffffu, *abort_flag)) {
         if (t == 0) {
           const uint32_t lbo = 128, sbo = (kKC / 8) * 128;
           const uint32_t d = tmem + (uint32_t)(st * NC);
@@ -333,16 +340,13 @@ __global__ void __launch_bounds__(kParts * kM, 1) colour_gemm_kernel(ColourGemmA
     }
     __syncthreads();
   }
-  // an expired wait: give the outstanding MMAs one more bounded wait before
-  // the tensor memory they write is released
-  for (int b = 0; b < 2; ++b)
-    if (outstanding[b]) mbar_wait(&bar[b], phase[b]);
-  // K-tile copies still in flight (only after an expired wait) land before the
-  // CTA's shared memory goes away
-  if (t == 0 && *abort_flag)
+  // after an expired wait: the MMAs and copies in flight, which the thread that
+  // issued them knows, get one more bounded wait before the CTA's tensor and shared
+  // memory go away
+  if (t == 0)
     for (int b = 0; b < 2; ++b) {
-      mbar_wait(&kbar[b], 0u);
-      mbar_wait(&kbar[b], 1u);
+      if (outstanding[b]) mbar_wait(&bar[b], phase[b]);
+      if (kpending[b]) mbar_wait(&kbar[b], kphase[b]);
     }
   fence_before();
   __syncthreads();
@@ -404,6 +408,7 @@ ColourTiles build_colour_tiles(const std::vector<int64_t>& K, int m) {
 size_t colour_gemm_smem(int nc) { return 2 * stage_bytes(nc) + 32 + 16 + (size_t)kM * 4 + 64; }
 
 cudaError_t launch_colour_gemm(const ColourGemmArgs& a, int num_sms, cudaStream_t s) {
+  static_assert(ColourGemmArgs().spin_limit == kSpinLimit, "the default of a launch");
   if (a.n_pairs <= 0) return cudaSuccess;
   if (a.nc < 32 || a.nc > 256 || a.nc % 32 != 0 || a.kp % kKC != 0 || a.np % a.nc != 0) return cudaErrorInvalidValue;
   // the kernel reads J in 16-byte vectors within rows of ldj >= m entries

@@ -1,5 +1,6 @@
 // Bounded waits of the tensor-core GEMMs that run out.  For every process given on
-// the command line the colour-amplitude GEMM runs on random diagram amplitudes with the usual limit, then with limits of 0 polls (every wait
+// the command line the colour-amplitude GEMM and the colour-sum GEMM run on random
+// diagram amplitudes with the usual limit, then with limits of 0 polls (every wait
 // expires at once), 1, 2, .. polls: each launch must end without an error, report
 // an expiry in its status word or none, and leave the next launch with the
 // usual limit to give the first one's results bit for bit.  Prints per process
@@ -73,6 +74,7 @@ int main(int argc, char** argv) {
     const Program P = build_program(pdg);
     const JampMap M = build_jamp_map(P);
     need(M.ok, "coefficients");
+    const ColourTiles T = build_colour_tiles(P.cf_jamp, P.n_jamp);
     const int64_t n = 64 * 3 * (int64_t)sms + 37;  // several tiles per CTA, a ragged last one
     const int64_t lda = (2 * n + 127) / 128 * 128;
     const int ldj = (P.n_jamp + 15) / 16 * 16;
@@ -86,6 +88,7 @@ int main(int argc, char** argv) {
         rowmax[r] = std::max(rowmax[r], std::fabs(v));
       }
     std::vector<float> J((size_t)2 * n * ldj), jabs((size_t)M.n_splits * n);
+    std::vector<double> pv(n);
     std::vector<int> status(1, 0);
     JampGemmArgs g;
     g.A = up(A);
@@ -104,6 +107,15 @@ int main(int argc, char** argv) {
     g.ldj = ldj;
     g.jabs = up(jabs);
     g.status = up(status);
+    ColourGemmArgs c;
+    c.J = up(J);  // the first launch's colour amplitudes (set below)
+    c.n_pairs = n;
+    c.m = P.n_jamp; c.ldj = ldj; c.kp = T.kp; c.np = T.np; c.nc = T.nc;
+    c.b_hi = up(T.hi);
+    c.b_lo = T.exact ? nullptr : up(T.lo);
+    c.inv_den = 1.0 / (double)P.cf_den;
+    c.pairval = up(pv);
+    c.status = g.status;
     auto launched = [&](cudaError_t e) {  // its status word
       ck(e, "launch");
       ck(cudaDeviceSynchronize(), "kernel");
@@ -124,18 +136,20 @@ int main(int argc, char** argv) {
       ++d;
     }
     std::vector<float> J0;
-    int expired = 0;
+    std::vector<double> pv0;
+    int expired[2] = {0, 0};
     for (uint32_t polls : {kDefault, 0u, kDefault, 1u, 2u, 3u, 4u, 8u, 16u, 64u, 256u, kDefault}) {
-      g.spin_limit = polls;
+      g.spin_limit = c.spin_limit = polls;
       const bool whole = polls == kDefault;
-      const int v = launched(launch_jamp_gemm(g, sms, nullptr));
+      int v = launched(launch_jamp_gemm(g, sms, nullptr));
       need(whole ? v == 0 : (v == 0 || v == 1), "status of the colour-amplitude GEMM");
       need(polls != 0 || v == 1, "no poll, no expiry (colour amplitudes)");
-      expired += v;
+      expired[0] += v;
       if (whole) {
         ck(cudaMemcpy(J.data(), g.J, J.size() * 4, cudaMemcpyDeviceToHost), "J");
         if (J0.empty()) {
           J0 = J;
+          ck(cudaMemcpy(const_cast<float*>(c.J), J0.data(), J0.size() * 4, cudaMemcpyHostToDevice), "J");
           for (int64_t p : {(int64_t)0, (int64_t)63, n / 2, n - 1})
             for (int ri = 0; ri < 2; ++ri)
               for (int a = 0; a < P.n_jamp; ++a) {
@@ -151,11 +165,20 @@ int main(int argc, char** argv) {
         }
         need(!std::memcmp(J.data(), J0.data(), J.size() * 4), "colour amplitudes after an expiry");
       }
+      v = launched(launch_colour_gemm(c, sms, nullptr));
+      need(whole ? v == 0 : (v == 0 || v == 1), "status of the colour-sum GEMM");
+      need(polls != 0 || v == 1, "no poll, no expiry (colour sum)");
+      expired[1] += v;
+      if (whole) {
+        ck(cudaMemcpy(pv.data(), c.pairval, n * 8, cudaMemcpyDeviceToHost), "pairval");
+        if (pv0.empty()) pv0 = pv;
+        need(!std::memcmp(pv.data(), pv0.data(), n * 8), "colour sum after an expiry");
+      }
     }
-    std::printf("%s %d\n", argv[arg], expired);
+    std::printf("%s %d %d\n", argv[arg], expired[0], expired[1]);
     for (const void* q : {(const void*)g.A, (const void*)g.rowmax, (const void*)g.tiles, (const void*)g.chunks, (const void*)g.split_begin,
-                          (const void*)g.kk_index, (const void*)g.kk_term, (const void*)g.J, (const void*)g.jabs,
-                          (const void*)g.status})
+                          (const void*)g.kk_index, (const void*)g.kk_term, (const void*)g.J, (const void*)g.jabs, (const void*)c.J,
+                          (const void*)c.b_hi, (const void*)c.b_lo, (const void*)c.pairval, (const void*)g.status})
       cudaFree(const_cast<void*>(q));
   }
   return faults ? 1 : 0;

@@ -1,8 +1,8 @@
-"""Waits of the tensor-core colour-amplitude GEMM (jamp_gemm.cu) that run out: a
+"""Waits of the tensor-core GEMMs (jamp_gemm.cu, colour_gemm.cu) that run out: a
 launch whose waits expire, at once or somewhere on the way, ends by itself with
 its status word set and leaves the context usable
 (tests/native/wait_expiry.cu).  One column block with derived columns, one
-without, and two blocks."""
+without, and two blocks; two CTAs per SM and one in the colour sum."""
 import os
 import subprocess
 
@@ -26,5 +26,5 @@ def test_expired_waits_end_the_launch(tmp_path):
     assert r.returncode == 0, r.stdout + r.stderr
     rows = [line.split() for line in r.stdout.splitlines()[1:]]
     assert [row[0] for row in rows] == procs
-    for name, expired in rows:
-        assert int(expired) >= 1, name
+    for name, amplitudes, total in rows:
+        assert int(amplitudes) >= 1 and int(total) >= 1, name
