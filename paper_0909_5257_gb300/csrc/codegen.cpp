@@ -51,9 +51,11 @@ void emit_body(std::ostringstream& o, const mea::Program& P, const std::string& 
   o << "  __device__ __forceinline__ static void run(const R* __restrict__ et, const R* __restrict__ mt,\n"
        "                                             uint32_t lam, R g, R gg, double inv_den, double& val,\n"
        "                                             float& kappa) {\n";
-  // Only the base of the colour amplitudes is accumulated (colour_base.h: half of
-  // them for pure gluons); the others are sums of its compensated sums at the
-  // end -- half the additions and half the registers.
+  // FP32: only the base of the colour amplitudes is accumulated (colour_base.h:
+  // half of them for pure gluons); the others are sums of its compensated sums at
+  // the end -- half the additions and half the registers.  The plain FP64 sums
+  // would lose digits that way where base amplitudes cancel, so FP64 accumulates
+  // every colour amplitude.
   const ColourBase base = find_colour_base(P);
   o << "    JSum<R> J[" << m << "];\n";
   o << "    float mass = 0.f;\n";
@@ -138,7 +140,7 @@ void emit_body(std::ostringstream& o, const mea::Program& P, const std::string& 
         for (uint32_t k = 0; k < op.col_count; ++k) {
           const ColEntry& c = P.col[op.col_begin + k];
           wsum += std::abs((int)c.re) + std::abs((int)c.im);
-          if ((int)c.alpha >= base.mb) continue;
+          if ((int)c.alpha >= base.mb) o << "      if constexpr (!std::is_same<R, float>::value)\n  ";
           if (cfac_real) {
             const int n = (int)c.re / cfac;
             if (n == 1 || n == -1)
@@ -160,11 +162,13 @@ void emit_body(std::ostringstream& o, const mea::Program& P, const std::string& 
     }
     if (!is_amp_op(op.type)) slot_op[op.out] = (int)i;
   }
+  if (base.mb < m) o << "    if constexpr (std::is_same<R, float>::value) {\n";
   for (int a = base.mb; a < m; ++a) {
     const uint16_t* ix = &base.index[3 * (a - base.mb)];
     for (int k = ix[0]; k < ix[2]; ++k)
-      o << "    " << (k < ix[1] ? "jadd" : "jsub") << "(J[" << a << "], J[" << base.term[k] << "]);\n";
+      o << "      " << (k < ix[1] ? "jadd" : "jsub") << "(J[" << a << "], J[" << base.term[k] << "]);\n";
   }
+  if (base.mb < m) o << "    }\n";
   // colour quadratic form with the integer colour matrix (symmetric)
   o << "    cx<R> F[" << m << "];\n    float jabs = 0.f;\n";
   const std::string scale = (cfac_real && cfac != 1) ? " * R(" + std::to_string(cfac) + ")" : "";

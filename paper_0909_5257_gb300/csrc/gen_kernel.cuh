@@ -64,17 +64,15 @@ __device__ __forceinline__ void jadd(JSum<double>& J, cx<double> a) {
   J.hi.r += a.r;
   J.hi.i += a.i;
 }
-// J += x, J -= x for another sum x
+// J += x, J -= x for another compensated sum x
 __device__ __forceinline__ void jadd(JSum<float>& J, const JSum<float>& x) {
   jadd(J, x.hi);
   J.lo = add2(J.lo, x.lo);
 }
-__device__ __forceinline__ void jadd(JSum<double>& J, const JSum<double>& x) { jadd(J, x.hi); }
 __device__ __forceinline__ void jsub(JSum<float>& J, const JSum<float>& x) {
   jadd(J, x.hi ^ 0x8000000080000000ull);
   J.lo = sub2(J.lo, x.lo);
 }
-__device__ __forceinline__ void jsub(JSum<double>& J, const JSum<double>& x) { jadd(J, cx<double>{-x.hi.r, -x.hi.i}); }
 
 template <typename R>
 __device__ __forceinline__ cx<R> neg(cx<R> a) {
