@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(kParts * kM, 1) colour_gemm_kernel(ColourGemmA
   auto wait_buf = [&](int b) -> bool {
     if (!outstanding[b]) return true;
     bool got = false;
-    if (!*abort_flag && !(got = mbar_wait(&bar[b], phase[b], g.spin_limit))) {
+    if (!*abort_flag && !(got = mbar_wait(&bar[b], phase[b]))) {
       atomicExch(abort_flag, 1);
       if (g.status) atomicExch(g.status, 1);
     }

@@ -30,7 +30,7 @@ struct ColourGemmArgs {
   double inv_den = 0;            // 1 / D
   double* pairval = nullptr;     // [n_pairs] output: J K J^* / D per pair
   int* status = nullptr;         // set to 1 when a bounded wait expired
-  uint32_t spin_limit = 1u << 19;  // polls of a bounded wait, tc::kSpinLimit (a test makes waits run out)
+  uint32_t spin_limit = 1u << 19;  // polls of the issuing thread's waits, tc::kSpinLimit (a test makes them run out)
 };
 
 // One-warp kernel whose bounded mbarrier wait expires (nothing arrives):

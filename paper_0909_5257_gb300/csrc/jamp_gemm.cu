@@ -276,11 +276,10 @@ __global__ void __launch_bounds__(kThreads, 1) jamp_gemm_kernel(JampGemmArgs g) 
       const int64_t pair = (int64_t)tile * kPairs + p;
       return pair < g.n_pairs ? __ldg(reinterpret_cast<const float2*>(g.rowmax) + pair) : make_float2(0.f, 0.f);
     };
-    // a bounded wait with one outcome for the warp
+    // a bounded wait with one outcome for the warp (its limit is a constant: read from
+    // the launch arguments it costs the conversion registers, 2 to 4 % of the stage)
     auto wait = [&](uint64_t* bar, uint32_t phase) {
-      const bool got = mbar_wait_abort(bar, phase, abort_flag, g.spin_limit);
-      if (!got) expired();
-      return __all_sync(0xffffffffu, got) != 0;
+      return __all_sync(0xffffffffu, mbar_wait_abort(bar, phase, abort_flag)) != 0;
     };
     uint32_t i = 0, tile_no = 0;
     Walk ahead, w, w_next;
@@ -362,6 +361,7 @@ __global__ void __launch_bounds__(kThreads, 1) jamp_gemm_kernel(JampGemmArgs g) 
       for (; ok && kc + 1 < n_kc; kc += 2) ok = step(pa0) && step(pa1);
       if (ok && kc < n_kc) ok = step(pa0);
       ok = ok && wait(done, tile_no & 1u);
+      if (!ok) expired();
       if (!vote_converters(ok)) break;  // also: row scales written
       fence_after();
 

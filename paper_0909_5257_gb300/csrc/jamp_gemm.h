@@ -61,7 +61,7 @@ struct JampGemmArgs {
   int ldj = 0;
   float* jabs = nullptr;          // [n_splits][n_pairs]: sum |J| over the split's columns
   int* status = nullptr;          // set to 1 when a bounded wait expired
-  uint32_t spin_limit = 1u << 19;  // polls of a bounded wait, tc::kSpinLimit (a test makes waits run out)
+  uint32_t spin_limit = 1u << 19;  // polls of the issuing thread's waits, tc::kSpinLimit (a test makes them run out)
 };
 
 cudaError_t launch_jamp_gemm(const JampGemmArgs& a, int num_sms, cudaStream_t s);

@@ -1,7 +1,8 @@
 // Bounded waits of the tensor-core GEMMs that run out.  For every process given on
 // the command line the colour-amplitude GEMM and the colour-sum GEMM run on random
-// diagram amplitudes with the usual limit, then with limits of 0 polls (every wait
-// expires at once), 1, 2, .. polls: each launch must end without an error, report
+// diagram amplitudes with the usual limit, then with limits of 0 polls (the first wait
+// of the threads that issue copies and MMAs expires at once, and the others give up
+// where they stand), 1, 2, .. polls: each launch must end without an error, report
 // an expiry in its status word or none, and leave the next launch with the
 // usual limit to give the first one's results bit for bit.  Prints per process
 // the launches with an expiry; exit status 1 on a fault.
