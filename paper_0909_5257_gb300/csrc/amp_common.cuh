@@ -251,12 +251,20 @@ __device__ __forceinline__ void tile_finish(const AmpLaunch& A, int t, int E, in
       if (evr < n) {
         int64_t gev = listed ? (int64_t)A.event_list[evr] : evr;
         double s = 0.0, wk = 0.0;
-        for (int hh = 0; hh < (A.paired ? 2 * H : H); ++hh) {
-          const int k = t * H + hel_lane(hh, H, A.paired);
-          double v = res[k];
+        // two plain loops: with the lane picked inside one (hel_lane), its registers
+        // cost the uu~>gg body the 96 that let 20 warps be resident
+        for (int hh = 0; hh < H; ++hh) {
+          double v = res[t * H + hh];
           s += v;
-          wk += v * (double)kap[k];
+          wk += v * (double)kap[t * H + hh];
         }
+        if (A.paired)
+#pragma unroll 1
+          for (int hh = H - 1; hh >= 0; --hh) {
+            double v = res[t * H + hh];
+            s += v;
+            wk += v * (double)kap[t * H + hh];
+          }
         double me = 0.25 * s;
         A.me2[gev] = me;
         uint8_t fl = inflags;

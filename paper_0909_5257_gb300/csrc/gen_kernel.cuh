@@ -15,18 +15,22 @@ namespace {
 constexpr int kGenMaxThreads = 256;
 
 // A colour amplitude under accumulation: FP64 plain, FP32 two-sum compensated
-// (lo collects the rounding errors) with its real and imaginary parts as one
-// packed pair, so that a compensated addition is 7 instructions instead of 14.
-// The FP32 pipe and the spills of the long body bound these kernels: packed
-// additions together with accumulating the base columns only take 2^20 events
-// of gg>ggg from 6.77 to 4.22 ms (168 registers) and from 8.03 to 5.25 ms
-// (128); gg>gg 0.66 ms either way (compute is not what it waits for).
-template <typename R>
+// (lo collects the rounding errors), PACKED with its real and imaginary parts as
+// one pair, so that a compensated addition is 7 instructions instead of 14 (the
+// same roundings).  The FP32 pipe and the spills of the long bodies bound these
+// kernels: packed additions together with accumulating the base columns only take
+// 2^20 events of gg>ggg from 6.77 to 4.22 ms (168 registers) and from 8.03 to
+// 5.25 ms (128).  Which bodies are packed: codegen.cpp.
+template <typename R, bool PACKED>
 struct JSum {
   cx<R> hi{R(0), R(0)};
 };
 template <>
-struct JSum<float> {
+struct JSum<float, false> {
+  cx<float> hi{0.f, 0.f}, lo{0.f, 0.f};
+};
+template <>
+struct JSum<float, true> {
   unsigned long long hi = 0, lo = 0;
 };
 
@@ -52,26 +56,42 @@ __device__ __forceinline__ unsigned long long sub2(unsigned long long a, unsigne
 }
 
 // J += a
-__device__ __forceinline__ void jadd(JSum<float>& J, unsigned long long a) {
+__device__ __forceinline__ void jadd(JSum<float, true>& J, unsigned long long a) {
   const unsigned long long s = add2(J.hi, a);
   const unsigned long long bp = sub2(s, J.hi);
   const unsigned long long e = add2(sub2(J.hi, sub2(s, bp)), sub2(a, bp));
   J.hi = s;
   J.lo = add2(J.lo, e);
 }
-__device__ __forceinline__ void jadd(JSum<float>& J, cx<float> a) { jadd(J, jpack(a)); }
-__device__ __forceinline__ void jadd(JSum<double>& J, cx<double> a) {
+__device__ __forceinline__ void jadd(JSum<float, true>& J, cx<float> a) { jadd(J, jpack(a)); }
+__device__ __forceinline__ void jadd(JSum<float, false>& J, cx<float> a) {
+  cx<float> s, e;
+  two_sum(J.hi.r, a.r, s.r, e.r);
+  two_sum(J.hi.i, a.i, s.i, e.i);
+  J.hi = s;
+  J.lo = J.lo + e;
+}
+template <bool PACKED>
+__device__ __forceinline__ void jadd(JSum<double, PACKED>& J, cx<double> a) {
   J.hi.r += a.r;
   J.hi.i += a.i;
 }
 // J += x, J -= x for another compensated sum x
-__device__ __forceinline__ void jadd(JSum<float>& J, const JSum<float>& x) {
+__device__ __forceinline__ void jadd(JSum<float, true>& J, const JSum<float, true>& x) {
   jadd(J, x.hi);
   J.lo = add2(J.lo, x.lo);
 }
-__device__ __forceinline__ void jsub(JSum<float>& J, const JSum<float>& x) {
+__device__ __forceinline__ void jsub(JSum<float, true>& J, const JSum<float, true>& x) {
   jadd(J, x.hi ^ 0x8000000080000000ull);
   J.lo = sub2(J.lo, x.lo);
+}
+__device__ __forceinline__ void jadd(JSum<float, false>& J, const JSum<float, false>& x) {
+  jadd(J, x.hi);
+  J.lo = J.lo + x.lo;
+}
+__device__ __forceinline__ void jsub(JSum<float, false>& J, const JSum<float, false>& x) {
+  jadd(J, -x.hi);
+  J.lo = J.lo - x.lo;
 }
 
 template <typename R>
@@ -79,8 +99,10 @@ __device__ __forceinline__ cx<R> neg(cx<R> a) {
   return cx<R>{-a.r, -a.i};
 }
 
-__device__ __forceinline__ cx<float> jfin(const JSum<float>& J) { return junpack(add2(J.hi, J.lo)); }
-__device__ __forceinline__ cx<double> jfin(const JSum<double>& J) { return J.hi; }
+__device__ __forceinline__ cx<float> jfin(const JSum<float, true>& J) { return junpack(add2(J.hi, J.lo)); }
+__device__ __forceinline__ cx<float> jfin(const JSum<float, false>& J) { return J.hi + J.lo; }
+template <bool PACKED>
+__device__ __forceinline__ cx<double> jfin(const JSum<double, PACKED>& J) { return J.hi; }
 
 // Register-cap variants: MINB resident CTAs of MAXT threads per SM cap a
 // thread at 65536 / (MAXT MINB) registers.  More registers spill less of the
@@ -88,7 +110,7 @@ __device__ __forceinline__ cx<double> jfin(const JSum<double>& J) { return J.hi;
 // depends on the body, so the FP32 bodies come at 128 (256 threads, MINB 2),
 // 85 (256, 3) and 168 (192, 2) registers and the autotuner picks.  Measured on
 // 2^20 events, ms at 168 / 128 / 85: gg>ggg 4.22 / 5.25 / 6.95, gg>gg 0.91 /
-// 0.76 / 0.66, uu~>gg 0.68 / 0.76 / 0.60.  The FP64 bodies come at 128.  A
+// 0.76 / 0.66, uu~>gg 0.69 / 0.64 / 0.61.  The FP64 bodies come at 128.  A
 // module that also held uncapped FP32 variants measured 25-45 % slower on the
 // same 128-register kernel, so none is built.
 template <typename R, typename Body, int MINB, int MAXT>

@@ -19,23 +19,25 @@
 #include "heget.cuh"
 
 // what gen_kernel.cuh gives the FP64 body; jfin reads the sums off
-template <typename R>
+template <typename R, bool PACKED>
 struct JSum {
   cx<R> hi{R(0), R(0)};
 };
 static std::vector<cx<double>> sums;
-inline void jadd(JSum<double>& J, cx<double> a) { J.hi = J.hi + a; }
+template <bool PACKED>
+void jadd(JSum<double, PACKED>& J, cx<double> a) { J.hi = J.hi + a; }
 template <typename R>
 inline cx<R> neg(cx<R> a) { return -a; }
-inline cx<double> jfin(const JSum<double>& J) {
+template <bool PACKED>
+cx<double> jfin(const JSum<double, PACKED>& J) {
   sums.push_back(J.hi);
   return J.hi;
 }
 // FP32 only (a body may name them where FP64 does not go)
-template <typename T>
-void jadd(JSum<T>&, const JSum<T>&);
-template <typename T>
-void jsub(JSum<T>&, const JSum<T>&);
+template <typename T, bool PACKED>
+void jadd(JSum<T, PACKED>&, const JSum<T, PACKED>&);
+template <typename T, bool PACKED>
+void jsub(JSum<T, PACKED>&, const JSum<T, PACKED>&);
 #include BODY_FILE
 
 using namespace mea;
