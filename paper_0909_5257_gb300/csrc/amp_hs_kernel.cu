@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(CAP == 0 ? 128 : 256, CAP == 0 ? 8 : 1)
   const int64_t n_tiles = (n + W - 1) / W;
   const float g = (float)P.g;
   const float gg = (float)(P.g * P.g);
-  const HsOpWords* ops = reinterpret_cast<const HsOpWords*>(P.ops);
+  const HsOpWords* ops = reinterpret_cast<const HsOpWords*>(P.ops_out);
   const int4* hs = reinterpret_cast<const int4*>(P.hs);
 
   for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
@@ -245,7 +245,6 @@ __global__ void __launch_bounds__(CAP == 0 ? 128 : 256, CAP == 0 ? 8 : 1)
       bool finite[NP];
 #pragma unroll
       for (int j = 0; j < NP; ++j) { mx_re[j] = 0.f; mx_im[j] = 0.f; mass[j] = 0.f; finite[j] = true; }
-      int d_amp = 0;
       // the records of op i + 1 are loaded while op i runs
       int4 nx0 = __ldg(&ops[0].v[0]), nx1 = __ldg(&ops[0].v[1]), nxq = __ldg(hs);
       for (int i = 0; i < P.n_ops; ++i) {
@@ -268,8 +267,8 @@ __global__ void __launch_bounds__(CAP == 0 ? 128 : 256, CAP == 0 ? 8 : 1)
           }
           __syncwarp();  // the variants are read by other lanes from here on
         } else {
-          const float wd = __ldg(P.amp_w + d_amp);
-          float* col = A.amp_out + (size_t)__ldg(P.amp_row + d_amp) * A.lda;
+          const float wd = __uint_as_float(op.col_count);
+          float* col = A.amp_out + (size_t)op.col_begin * A.lda;
 #pragma unroll
           for (int j = 0; j < NP; ++j) {
             const int h = lane + 32 * j;
@@ -285,7 +284,6 @@ __global__ void __launch_bounds__(CAP == 0 ? 128 : 256, CAP == 0 ? 8 : 1)
               mass[j] += wd * (ar + ai);
             }
           }
-          ++d_amp;
         }
       }
       const float nan = __int_as_float(0x7fc00000);
@@ -428,7 +426,6 @@ __global__ void __launch_bounds__(512) amp_hsp_kernel(const DevProgram P, const 
       const int64_t pair = ev * H + h;
       float mx_re = 0.f, mx_im = 0.f, mass = 0.f;
       bool finite = true;
-      int d_amp = 0;
       W4<float> tr;
       for (int k = 0; k < 4; ++k) tr.c[k] = {0.f, 0.f};
       int4 nx0 = __ldg(&mops[0].v[0]), nx1 = __ldg(&mops[0].v[1]), nxq = __ldg(mrec);
@@ -449,13 +446,12 @@ __global__ void __launch_bounds__(512) amp_hsp_kernel(const DevProgram P, const 
           tr = hs_produce(op, P, x, et, mt, g, gg);
         } else {
           const cx<float> amp = hs_amplitude(op, x, mt, g, gg);
-          *reinterpret_cast<float2*>(A.amp_out + (size_t)__ldg(P.amp_row + d_amp) * A.lda + 2 * pair) = make_float2(amp.r, amp.i);
+          *reinterpret_cast<float2*>(A.amp_out + (size_t)op.col_begin * A.lda + 2 * pair) = make_float2(amp.r, amp.i);
           const float a_r = fabsf(amp.r), a_i = fabsf(amp.i);
           finite = finite && isfinite(a_r) && isfinite(a_i);
           mx_re = fmaxf(mx_re, a_r);
           mx_im = fmaxf(mx_im, a_i);
-          mass += __ldg(P.amp_w + d_amp) * (a_r + a_i);
-          ++d_amp;
+          mass += __uint_as_float(op.col_count) * (a_r + a_i);
         }
       }
       const float nan = __int_as_float(0x7fc00000);

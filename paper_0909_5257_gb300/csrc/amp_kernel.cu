@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(kMaxThreads) amp_kernel(const DevProgram P, co
   const int64_t n_tiles = (n + E - 1) / E;
   const R g = (R)P.g;
   const R gg = (R)(P.g * P.g);
-  const OpWords* ops = reinterpret_cast<const OpWords*>(P.ops);
+  const OpWords* ops = reinterpret_cast<const OpWords*>(AOUT ? P.ops_out : P.ops);
 
   for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
     const int64_t ev0 = tile * E;
@@ -307,24 +307,22 @@ __global__ void __launch_bounds__(kMaxThreads) amp_kernel(const DevProgram P, co
       if (!AOUT)
         for (int a = 0; a < m * JW; ++a) jam[(size_t)a * L + t] = (R)0;
       float abs_mass = 0.f;  // sum of |c A| over all colour entries (FP32 indicator)
-      // amplitude output: diagram ordinal, row maxima of |Re A|, |Im A|, finiteness
+      // amplitude output: row maxima of |Re A|, |Im A|, finiteness
       const int64_t pair = ev * H + h;
-      int d_amp = 0;
       float mx_re = 0.f, mx_im = 0.f;
       bool finite_amps = true;
 
-      // one diagram amplitude: to the tensor-core stage (AOUT) or into the
-      // colour amplitudes through its colour entries
+      // one diagram amplitude: to the tensor-core stage (AOUT, its row and weight) or
+      // into the colour amplitudes through its colour entries
       auto take_amp = [&](uint32_t col_begin, uint32_t col_count, const cx<R>& amp) {
         if (AOUT) {
-          float2* dst = reinterpret_cast<float2*>(A.amp_out + (size_t)__ldg(P.amp_row + d_amp) * A.lda + 2 * pair);
+          float2* dst = reinterpret_cast<float2*>(A.amp_out + (size_t)col_begin * A.lda + 2 * pair);
           *dst = make_float2((float)amp.r, (float)amp.i);
           const float ar = fabsf((float)amp.r), ai = fabsf((float)amp.i);
           finite_amps = finite_amps && isfinite(ar) && isfinite(ai);
           mx_re = fmaxf(mx_re, ar);
           mx_im = fmaxf(mx_im, ai);
-          abs_mass += __ldg(P.amp_w + d_amp) * (ar + ai);
-          ++d_amp;
+          abs_mass += __uint_as_float(col_count) * (ar + ai);
         } else {
           const ColEntry* ce = P.col + col_begin;
           for (uint32_t k = 0; k < col_count; ++k) {

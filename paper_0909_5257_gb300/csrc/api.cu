@@ -582,10 +582,9 @@ mea_status mea_create_process(const int* pdg, int n_ext, const mea_options* opts
     P->jmap = mea::build_jamp_map(G);
     if (P->jmap.ok) {
       const __half* dt = nullptr;
-      const float* dw = nullptr;
-      const int* dr = nullptr;
-      if ((e = upload(P, P->jmap.tiles, &dt)) != cudaSuccess || (e = upload(P, P->jmap.weight, &dw)) != cudaSuccess ||
-          (e = upload(P, P->jmap.row, &dr)) != cudaSuccess || (e = upload(P, P->jmap.chunks, &P->jmap_chunks)) != cudaSuccess ||
+      if ((e = upload(P, P->jmap.tiles, &dt)) != cudaSuccess ||
+          (e = upload(P, mea::amplitude_output_ops(G.ops, P->jmap), &D.ops_out)) != cudaSuccess ||
+          (e = upload(P, P->jmap.chunks, &P->jmap_chunks)) != cudaSuccess ||
           (e = upload(P, P->jmap.split_begin, &P->jmap_begin)) != cudaSuccess ||
           (e = upload(P, P->jmap.kk_index, &P->jmap_kk_index)) != cudaSuccess ||
           (e = upload(P, P->jmap.kk_term, &P->jmap_kk_term)) != cudaSuccess) {
@@ -593,8 +592,6 @@ mea_status mea_create_process(const int* pdg, int n_ext, const mea_options* opts
         return fail(MEA_E_CUDA, std::string("mea_create_process: ") + cudaGetErrorString(e));
       }
       P->jmap_tiles = dt;
-      D.amp_w = dw;
-      D.amp_row = dr;
       std::vector<__half>().swap(P->jmap.tiles);
     }
   }
@@ -680,7 +677,7 @@ mea_status mea_create_process(const int* pdg, int n_ext, const mea_options* opts
     const mea::HsOp *dr = nullptr, *dmr = nullptr;
     const mea::Op* dmo = nullptr;
     if ((e = upload(P, P->hsp.tasks, &dt)) != cudaSuccess || (e = upload(P, P->hsp.rec, &dr)) != cudaSuccess ||
-        (e = upload(P, P->hsp.main_ops, &dmo)) != cudaSuccess || (e = upload(P, P->hsp.main_rec, &dmr)) != cudaSuccess) {
+        (e = upload(P, mea::amplitude_output_ops(P->hsp.main_ops, P->jmap), &dmo)) != cudaSuccess || (e = upload(P, P->hsp.main_rec, &dmr)) != cudaSuccess) {
       destroy(P);
       return fail(MEA_E_CUDA, std::string("mea_create_process: ") + cudaGetErrorString(e));
     }

@@ -52,6 +52,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstdlib>
+#include <cstring>
 #include <numeric>
 
 #include "colour_base.h"
@@ -569,6 +570,17 @@ JampMap build_jamp_map(const Program& p) {
   }
   M.ok = q >= 8;  // digit truncation below 2^-27 of the row maximum
   return M;
+}
+
+std::vector<Op> amplitude_output_ops(std::vector<Op> ops, const JampMap& m) {
+  size_t d = 0;
+  for (Op& op : ops) {
+    if (!is_amp_op(op.type)) continue;
+    op.col_begin = (uint32_t)m.row.at(d);
+    std::memcpy(&op.col_count, &m.weight.at(d), sizeof op.col_count);
+    ++d;
+  }
+  return ops;
 }
 
 size_t jamp_gemm_smem(const JampGemmArgs& a) {

@@ -43,6 +43,10 @@ struct JampMap {
 
 JampMap build_jamp_map(const Program& p);
 
+// `ops` (all amplitudes of the program, in its order) with every amplitude's row
+// and weight bits in its colour fields (DevProgram::ops_out).
+std::vector<Op> amplitude_output_ops(std::vector<Op> ops, const JampMap& m);
+
 struct JampGemmArgs {
   const float* A = nullptr;      // [kd][lda]: A[d*lda + 2p] = Re A_d, [.. + 1] = Im A_d of pair p
   int64_t lda = 0;

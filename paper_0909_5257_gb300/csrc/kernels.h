@@ -53,8 +53,10 @@ struct DevProgram {
   double g = 0;                       // g_s
   const GenEntry* gen = nullptr;      // straight-line kernel of this process, if emitted
   int gen_forced = -1;                // FP32 variant pinned by mea_options.kernel_variant (-1: free)
-  const float* amp_w = nullptr;       // [n_diagrams] sum_alpha |c_alpha d| (amplitude-output mode)
-  const int* amp_row = nullptr;       // [n_diagrams] row of each diagram in the amplitude buffer
+  // amplitude-output mode: the program with, in an amplitude's col_begin and
+  // col_count, its row in the amplitude buffer and the bits of its weight
+  // sum_alpha |c_alpha d| (a float), so that both come with the op
+  const Op* ops_out = nullptr;
   const HsOp* hs = nullptr;           // helicity-shared layout of the program (helshare.h), or null
   int hs_arena = 0;                   // its variants per event
   bool hs_only = false;               // amplitude-output mode: plan and tune the helicity-shared kernel only
@@ -63,7 +65,7 @@ struct DevProgram {
   int hsp_level_end[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   int hsp_levels = 0;
   const HsOp* hsp_rec = nullptr;        // [n_ops] records of the whole program
-  const Op* hsp_main_ops = nullptr;     // the per-lane ops
+  const Op* hsp_main_ops = nullptr;     // the per-lane ops, amplitudes as in ops_out
   const HsOp* hsp_main_rec = nullptr;
   int hsp_n_main = 0;
   int hsp_area = 0;                     // prologue variants per event
@@ -114,7 +116,7 @@ struct AmpLaunch {
   float* pair_kappa = nullptr;        // per-pair indicator (see amp_out)
   uint8_t* ev_flags = nullptr;        // amplitude-output mode: per-event input-check bits out;
                                       //   finish_kernel ORs them into the flags
-  float* amp_out = nullptr;           // amplitude-output mode: A[amp_row[d]][lda], (Re, Im) of pair p at 2p, 2p+1;
+  float* amp_out = nullptr;           // amplitude-output mode: A[row of d][lda], (Re, Im) of pair p at 2p, 2p+1;
   int64_t lda = 0;                    //   pair_kappa then receives sum_d w_d |A_d| and
   float* amp_rowmax = nullptr;        //   amp_rowmax[2p], [2p+1] the row maxima of |Re A|, |Im A|
   float* jamp_scratch = nullptr;      // global colour-amplitude accumulators when not in SMEM
