@@ -621,7 +621,7 @@ cudaError_t launch_amp_hsp(const DevProgram& p, const AmpConfig& c, const AmpLau
   const void* k = c.slots_in_smem ? (const void*)amp_hsp_kernel<true> : (const void*)amp_hsp_kernel<false>;
   cudaError_t e = ensure_dynamic_smem(k, c.smem);
   if (e != cudaSuccess) return e;
-  if (cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, carveout_percent(c)) != cudaSuccess)
+  if (cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, carveout_percent(p, c)) != cudaSuccess)
     cudaGetLastError();
   if (c.slots_in_smem) amp_hsp_kernel<true><<<c.grid, c.threads, c.smem, s>>>(p, a, c);
   else amp_hsp_kernel<false><<<c.grid, c.threads, c.smem, s>>>(p, a, c);
@@ -636,7 +636,7 @@ cudaError_t launch_amp_hs(const DevProgram& p, const AmpConfig& c, const AmpLaun
   const void* k = hs_kernel_for(c.H, c.regvar);
   cudaError_t e = ensure_dynamic_smem(k, c.smem);
   if (e != cudaSuccess) return e;
-  if (cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, carveout_percent(c)) != cudaSuccess)
+  if (cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, carveout_percent(p, c)) != cudaSuccess)
     cudaGetLastError();
   if (c.regvar == 0) hs_launch<0>(p, c, a, s);
   else hs_launch<1>(p, c, a, s);

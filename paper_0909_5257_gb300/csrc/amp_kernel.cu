@@ -492,16 +492,6 @@ static int gen_body_variant(const DevProgram& p, int cap) {
   return 2 * cap + (p.family == FAM_TWO_LINES && p.n_ext == 5 && cap == 1 ? 1 : 0);
 }
 
-int sm_count() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    n = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0 ? v : 1;
-  }
-  return n;
-}
-
 size_t gen_smem(const DevProgram& p, int E, int threads, size_t real) {
   return (((size_t)E * event_table_stride(p.n_ext, p.n_masks) * real + 7) & ~size_t(7)) + (size_t)threads * 16 + 16;
 }
@@ -516,7 +506,7 @@ size_t gen_smem(const DevProgram& p, int E, int threads, size_t real) {
 // -> 20.9 us, gg>gg 23.1 -> 15.5, uu~>gg 18.8 -> 15.0, gg>ggg 35.5 -> 31.2,
 // uu>uug 21.9 -> 18.7; gg>gg in FP64 54.0 -> 41.6.
 AmpConfig gen_spread(const DevProgram& p, const AmpConfig& plan, int64_t n_events, size_t real) {
-  const int64_t sms = sm_count();
+  const int64_t sms = p.num_sms;
   const int E = (int)std::max<int64_t>(1, (n_events + sms - 1) / sms);
   if (E >= plan.E_cta) return plan;
   AmpConfig c = plan;
@@ -818,17 +808,9 @@ size_t slot_scratch_bytes_needed(const DevProgram& p, bool fp64, const AmpConfig
   return (size_t)c.grid * p.n_slots * 8 * c.threads * (fp64 ? sizeof(double) : sizeof(float));
 }
 
-int carveout_percent(const AmpConfig& c) {
-  static int smem_sm = 0;
-  if (smem_sm == 0) {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess || v <= 0)
-      v = 228 * 1024;
-    smem_sm = v;
-  }
+int carveout_percent(const DevProgram& p, const AmpConfig& c) {
   const double need = (double)std::max(1, c.per_sm) * ((double)c.smem + 1024.0);  // 1 KB reserved per CTA
-  return std::max(0, std::min(100, (int)std::ceil(100.0 * need / smem_sm) + 1));
+  return std::max(0, std::min(100, (int)std::ceil(100.0 * need / p.smem_sm) + 1));
 }
 
 template <typename R, bool J, bool S, bool O = false, bool F = false>
@@ -837,7 +819,7 @@ static cudaError_t launch_one(const DevProgram& p, const AmpConfig& c, const Amp
   if (e != cudaSuccess) return e;
   // the carveout is a preference: a value the driver refuses leaves the launch valid
   if (cudaFuncSetAttribute(amp_kernel<R, J, S, O, F>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                           carveout_percent(c)) != cudaSuccess)
+                           carveout_percent(p, c)) != cudaSuccess)
     cudaGetLastError();
   amp_kernel<R, J, S, O, F><<<c.grid, c.threads, c.smem, s>>>(p, a, c);
   return cudaGetLastError();

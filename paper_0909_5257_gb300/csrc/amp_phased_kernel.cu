@@ -445,7 +445,7 @@ cudaError_t launch_amp_phased(const DevProgram& p, const AmpConfig& c, const Amp
     return cudaErrorInvalidConfiguration;
   cudaError_t e = ensure_dynamic_smem((const void*)amp_phased_kernel, c.smem);
   if (e != cudaSuccess) return e;
-  if (cudaFuncSetAttribute(amp_phased_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, carveout_percent(c)) !=
+  if (cudaFuncSetAttribute(amp_phased_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, carveout_percent(p, c)) !=
       cudaSuccess)
     cudaGetLastError();
   amp_phased_kernel<<<c.grid, c.threads, c.smem, s>>>(p, a, c);

@@ -539,6 +539,8 @@ mea_status mea_create_process(const int* pdg, int n_ext, const mea_options* opts
     return fail(e == cudaErrorMemoryAllocation ? MEA_E_NOMEM : MEA_E_CUDA,
                 std::string("mea_create_process: ") + cudaGetErrorString(e));
   }
+  D.num_sms = P->num_sms;
+  D.smem_sm = (int)P->smem_per_sm;
   D.ops = dops;
   D.n_ops = (int)G.ops.size();
   D.col = dcol;

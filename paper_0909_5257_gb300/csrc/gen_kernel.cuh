@@ -176,7 +176,7 @@ void gen_launch_v(const DevProgram& p, const AmpConfig& plan, const AmpLaunch& a
   if (ensure_dynamic_smem((const void*)k, c.smem) != cudaSuccess) return;
   // the carveout is a preference: a value the driver refuses leaves the launch valid.  The
   // plan's, so that calls of several sizes do not reconfigure the SMs (uu~>ggg, 4096 events: 29 -> 37 us).
-  if (cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, carveout_percent(plan)) != cudaSuccess)
+  if (cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, carveout_percent(p, plan)) != cudaSuccess)
     cudaGetLastError();
   k<<<c.grid, c.threads, c.smem, s>>>(p, a, c);
 }

@@ -34,6 +34,7 @@ const GenEntry* find_generated(const int* pdg, int n_ext);
 
 // Device copy of a process program (all pointers are device memory).
 struct DevProgram {
+  int num_sms = 0, smem_sm = 0;       // of the device that the process was created on: SMs, shared memory of one (bytes)
   const Op* ops = nullptr;
   int n_ops = 0;
   const ColEntry* col = nullptr;
@@ -148,9 +149,7 @@ struct AmpConfig {
 // holds per_sm CTAs of smem bytes each and leaves the rest as L1: the
 // straight-line kernels spill and the interpreter keeps wavefunction slots in
 // global memory, both of which live in L1.
-int carveout_percent(const AmpConfig& c);
-
-int sm_count();  // of the current device
+int carveout_percent(const DevProgram& p, const AmpConfig& c);
 
 // The straight-line kernels' tile for a call of n_events (dynamic shared memory for a real of that many bytes).
 AmpConfig gen_spread(const DevProgram& p, const AmpConfig& plan, int64_t n_events, size_t real);

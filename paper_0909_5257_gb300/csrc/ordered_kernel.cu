@@ -184,13 +184,13 @@ cudaError_t launch_ordered(const DevProgram& p, const AmpConfig& c, const AmpLau
   // fewer events than the tiles of a full grid hold: smaller tiles on more CTAs
   int E = c.E_cta, grid = c.grid;
   if (!a.event_list && c.slots_in_smem && c.jamp_in_smem) {
-    const int64_t full = (int64_t)c.per_sm * sm_count();
+    const int64_t full = (int64_t)c.per_sm * p.num_sms;
     E = (int)std::max<int64_t>(1, std::min<int64_t>(E, (a.n_events + full - 1) / full));
     grid = (int)std::min<int64_t>(full, (a.n_events + E - 1) / E);
   }
   cudaError_t e = ensure_dynamic_smem((const void*)ordered_kernel, c.smem);
   if (e != cudaSuccess) return e;
-  if (cudaFuncSetAttribute(ordered_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, carveout_percent(c)) != cudaSuccess)
+  if (cudaFuncSetAttribute(ordered_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, carveout_percent(p, c)) != cudaSuccess)
     cudaGetLastError();
   ordered_kernel<<<grid, c.threads, ord_smem(p, E, c.slots_in_smem, c.jamp_in_smem), s>>>(p, a, E, c.slots_in_smem, c.jamp_in_smem);
   return cudaGetLastError();
