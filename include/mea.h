@@ -116,8 +116,16 @@ typedef struct {
                             autotuner choosing its CTA size) for MEA_HEL_SUM_NONZERO
                             of processes with 6 or 7 partons, else the autotuner's
                             choice (untuned: the per-lane interpreter) among the
-                            kernels below; all apply the same operations to the
-                            same inputs (bit-identical results); 1 per-lane
+                            kernels below.  All apply the same operations to the
+                            same inputs: the diagram amplitudes, and with them me2
+                            of an event that stays on the mixed path, are the same
+                            bits in every mode (checked for each build by the tests:
+                            the compiler chooses the roundings of all but the phased
+                            kernel).  The cancellation indicator is not: the phased
+                            kernel adds its magnitudes in another order, so an event
+                            whose indicator lies within rounding of flag_threshold
+                            can be flagged, and re-evaluated in FP64, in one mode and
+                            not in another.  1 per-lane
                             interpreter (one lane per event and helicity
                             combination) only, tuned with and without forwarding
                             each op's output to the next op in registers; 2
