@@ -214,6 +214,26 @@ mea_status mea_colour_matrix(mea_process_t proc, int64_t *num, int64_t *den);
  * host buffer of capacity cap rows; *n_hel receives the count. */
 mea_status mea_helicities(mea_process_t proc, int8_t *hel, int cap, int *n_hel);
 
+/* Diagnostics, no counterpart in the paper: which kernels the next
+ * MEA_HEL_SUM_NONZERO evaluation runs (a layout that a process does not have
+ * makes it fall back on another kernel with the same results), and what the
+ * tensor-core path's colour-amplitude GEMM contracts.  MEA_E_UNSUPPORTED on a
+ * host-only handle. */
+typedef struct {
+  int helicity_lanes;    /* helicity combinations evaluated (one of each flipped pair
+                            for pure gluons) */
+  int fp64_recursion;    /* FP64 path: 1 the colour-ordered recursion, 0 the diagrams */
+  int mixed_path;        /* mixed path: 0 straight-line kernel, 1 table-driven
+                            interpreter, 2 tensor-core path */
+  int amplitude_kernel;  /* tensor-core path: 0 per-lane, 1 helicity-shared, 2 split,
+                            3 phased (as mea_tune_result.helicity_shared); else -1 */
+  int gemm_base;         /* colour amplitudes contracted (the others are sums of them) */
+  int gemm_columns;      /* columns per block of them, padded */
+  int gemm_chunks;       /* (block, 64 diagrams) tiles contracted: those with a coefficient */
+  double phased_flops_per_event; /* operations of the phased kernel; 0 without its layout */
+} mea_kernel_info;
+mea_status mea_process_kernels(mea_process_t proc, mea_kernel_info *out);
+
 mea_status mea_destroy_process(mea_process_t proc);
 
 /* Synchronise `stream` and report whether any bounded device wait of this

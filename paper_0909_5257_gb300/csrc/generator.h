@@ -19,6 +19,7 @@
 #pragma once
 #include <array>
 #include <cstdint>
+#include <stdexcept>
 #include <string>
 #include <utility>
 #include <vector>
@@ -42,6 +43,12 @@ enum OpType : uint8_t {
   OP_PGGGG = 12, // vertex partial G(in[0], in[1], in[2]) of ggggxx (heget.cuh gggg_part)
   OP_PIOV = 13,  // vertex partial of iovxx0, leg = free argument (0 fi, 1 fo, 2 V):
                  // (fo, V), (fi, V) or (fi, fo) in in[0], in[1]
+};
+
+// A kernel layout that a process does not have (too many rows, values that do not
+// fit, ..): the caller falls back on another kernel.
+struct LayoutError : std::runtime_error {
+  using std::runtime_error::runtime_error;
 };
 
 // Amplitude operations (one per Feynman diagram, in diagram-ordinal order).

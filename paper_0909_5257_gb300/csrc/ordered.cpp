@@ -16,7 +16,7 @@ namespace {
 typedef std::vector<int> Word;  // letters
 
 void check(bool ok, const char* why) {
-  if (!ok) throw std::runtime_error(std::string("ordered recursion: ") + why);
+  if (!ok) throw LayoutError(std::string("ordered recursion: ") + why);
 }
 
 struct Val {

@@ -100,7 +100,7 @@ struct OrdProgram {
   double norm = 0;                 // |M|^2 = norm g^(2n-4) sum_h J K J^*, parity and averages included
 };
 
-// Throws std::runtime_error when a word needs a momentum the program's event
+// Throws LayoutError when a word needs a momentum the program's event
 // table does not hold or a table does not fit its type.
 OrdProgram build_ordered(const Program& P);
 

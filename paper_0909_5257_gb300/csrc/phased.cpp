@@ -45,7 +45,7 @@ struct Costed {
 };
 
 void check(bool ok, const char* why) {
-  if (!ok) throw std::runtime_error(std::string("phased layout: ") + why);
+  if (!ok) throw LayoutError(std::string("phased layout: ") + why);
 }
 
 }  // namespace
@@ -98,6 +98,8 @@ PhProgram build_phased(const Program& P, const HelLanes& lanes, const std::vecto
       holder.at(op.out) = i;
     }
   }
+  for (int i = 0; i < n_ops; ++i)
+    if (ordinal[i] >= 0) Q.flops += (double)H * op_flop_cost(P.ops[i]);
   check(n_amp < 0x10000 && weight.size() == (size_t)n_amp && row.size() == weight.size(),
         "diagram ordinals of 16 bits");
 
@@ -209,6 +211,7 @@ PhProgram build_phased(const Program& P, const HelLanes& lanes, const std::vecto
       for (int v = 0; v < (int)u.size(); ++v) {
         if (!u[v]) continue;
         const uint32_t lam = pdep8(v, legs[i]);
+        Q.flops += op_flop_cost(op);
         PhItem it{};
         it.out = (uint16_t)(off[i] + v);
         for (int k = 0; k < n_in; ++k) {
@@ -336,6 +339,7 @@ PhProgram build_phased(const Program& P, const HelLanes& lanes, const std::vecto
       for (int v = 0; v < (int)u.size(); ++v)
         if (u[v]) vs.push_back(v);
       check(!vs.empty() && vs.size() <= 32, "variants of a fused current");
+      for (int i : g.second) Q.flops += (double)vs.size() * op_flop_cost(P.ops[fused_amp[i]]);
       int lg = 0;
       while ((1 << lg) < (int)vs.size()) ++lg;
       if (!set_index.count(S)) {

@@ -115,10 +115,11 @@ struct PhProgram {
   int area = 0;                    // variants per event
   int H = 0;
   double cost = 0;                 // estimated warp instructions per event
+  double flops = 0;                // of the evaluated operations per event (op_flop_cost)
 };
 
 // lanes: the helicity combinations; weight[d]: sum of the colour coefficients' magnitudes of diagram d
-// (JampMap::weight), row[d] its row in the amplitude buffer (JampMap::row).  Throws std::runtime_error when the program does not have
+// (JampMap::weight), row[d] its row in the amplitude buffer (JampMap::row).  Throws LayoutError when the program does not have
 // the structure above or its area exceeds max_area variants.
 PhProgram build_phased(const Program& P, const HelLanes& lanes, const std::vector<float>& weight,
                        const std::vector<int>& row, int max_area);

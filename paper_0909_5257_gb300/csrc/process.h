@@ -61,6 +61,7 @@ struct mea_process_s {
   mea::HsSplitProgram hsp;  // split layout of prog (valid when hsp_ok)
   bool hsp_ok = false;
   mea::PhProgram ph;               // phased layout (until uploaded)
+  double ph_flops = 0;             // its operations per event
   std::vector<mea::AmpConfig> ph_cands;  // launch shapes of the phased kernel
   mea::DevProgram dev;
   mea_options opts;

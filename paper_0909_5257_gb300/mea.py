@@ -52,6 +52,12 @@ class ProcessInfo(ctypes.Structure):
                 ("hsp_flops_per_event", ctypes.c_double)]
 
 
+class KernelInfo(ctypes.Structure):
+    _fields_ = [("helicity_lanes", ctypes.c_int), ("fp64_recursion", ctypes.c_int), ("mixed_path", ctypes.c_int),
+                ("amplitude_kernel", ctypes.c_int), ("gemm_base", ctypes.c_int), ("gemm_columns", ctypes.c_int),
+                ("gemm_chunks", ctypes.c_int), ("phased_flops_per_event", ctypes.c_double)]
+
+
 class TuneResult(ctypes.Structure):
     _fields_ = [("threads", ctypes.c_int), ("events_per_cta", ctypes.c_int), ("grid", ctypes.c_int),
                 ("colour_amps_in_shared", ctypes.c_int), ("slots_in_shared", ctypes.c_int),
@@ -99,6 +105,7 @@ def load(path: str | None = None):
             lib.mea_create_process.argtypes = [vp, i32, vp, vp]
             lib.mea_create_process_host_only.argtypes = [vp, i32, vp, vp]
             lib.mea_process_info.argtypes = [vp, vp]
+            lib.mea_process_kernels.argtypes = [vp, vp]
             lib.mea_colour_matrix.argtypes = [vp, vp, vp]
             lib.mea_helicities.argtypes = [vp, vp, i32, vp]
             lib.mea_destroy_process.argtypes = [vp]
@@ -125,7 +132,7 @@ def load(path: str | None = None):
             lib.mea_server_destroy.argtypes = [vp]
             lib.mea_last_error.restype = ctypes.c_char_p
             lib.mea_kernel_launch_count.restype = ctypes.c_uint64
-            for name in ("mea_create_process", "mea_create_process_host_only", "mea_process_info",
+            for name in ("mea_create_process", "mea_create_process_host_only", "mea_process_info", "mea_process_kernels",
                          "mea_colour_matrix", "mea_helicities", "mea_destroy_process", "mea_evaluate",
                          "mea_evaluate_host", "mea_evaluate_noalloc", "mea_generate_phase_space",
                          "mea_check_status", "mea_autotune", "mea_batch_create", "mea_batch_launch",
@@ -226,6 +233,12 @@ class Process:
             self.close()
         except Exception:
             pass
+
+    def kernels(self):
+        """Which kernels the next helicity-summed evaluation runs (mea_process_kernels)."""
+        k = KernelInfo()
+        _check(load().mea_process_kernels(self._h, ctypes.byref(k)))
+        return {name: getattr(k, name) for name, _ in KernelInfo._fields_}
 
     @property
     def n_colour(self):
