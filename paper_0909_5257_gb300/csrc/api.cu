@@ -749,6 +749,7 @@ mea_status mea_create_process_host_only(const int* pdg, int n_ext, const mea_opt
     destroy(P);
     return fail(MEA_E_UNSUPPORTED, std::string("mea_create_process_host_only: ") + e.what());
   }
+  P->lanes = mea::helicity_lanes(P->prog);
   try {
     P->hs = mea::build_helicity_shared(P->prog, P->prog.n_hel);
     P->hs_ok = true;

@@ -123,6 +123,8 @@ mea_status autotune_locked(mea_process_s* P, const double* mom, int64_t n, mea_p
 // Heuristic launch plan of this process for n events (cached per precision,
 // path and helicity count); dp is P->dev or its tensor-path copy.
 AmpConfig cached_plan(mea_process_s* P, const DevProgram& dp, bool fp64, bool tc, int H, int64_t n);
+// Estimated cost of an event (FLOPs of the mixed path; dispatch order and chunk sizes of the server).
+double request_cost(const mea_process_s* P, mea_prec_mode prec);
 // Device scratch bytes an evaluation of n events would hold (admission control).
 size_t scratch_estimate(mea_process_s* P, int64_t n, mea_prec_mode prec);
 }  // namespace mea

@@ -44,7 +44,10 @@ using Clock = std::chrono::steady_clock;
 constexpr double kChunkFlop = 1e11;    // target device work of one chunk
 constexpr int64_t kChunkQuantum = 128; // chunk sizes are multiples of this (or the whole request)
 constexpr double kAging = 0.25;        // priority gained per second waited, in seconds of work
-constexpr double kFp64Cost = 24.0;     // FP64 path cost per FLOP relative to the mixed path (measured 19-28)
+// FP64 path cost relative to the mixed path: whole calls of the five-jet processes
+// measured 8.1 (gg>5g), 8.9 (uu~>5g) and 9.8 (uu>uu+3g), of the four-jet ones 4.6 to
+// 9.6, below that 2.5 to 22
+constexpr double kFp64Cost = 9.0;
 constexpr double kInitialRate = 1e13;  // FLOP/s assumed until the server has measured its own
 
 struct SrvReq {
@@ -88,6 +91,14 @@ struct ProcState {
 };
 
 }  // namespace
+
+// Cost of an event: the process's operation count, amplitudes and colour sum, over the
+// helicity combinations that are evaluated, the FP64 path weighted by its measured
+// slowdown.
+double mea::request_cost(const mea_process_s* P, mea_prec_mode prec) {
+  const double m = P->prog.n_jamp, per_combination = P->prog.flops_per_hel + 4.0 * m * m;
+  return std::max(1.0, per_combination * std::max(1, P->lanes.n) * (prec == MEA_PREC_FP64 ? kFp64Cost : 1.0));
+}
 
 struct mea_server_s {
   size_t budget = 0, reserved = 0;  // reserved: sum of the processes' commitments
@@ -321,10 +332,7 @@ mea_status mea_server_submit(mea_server_t S, mea_process_t P, const double* mom,
   r->prec = prec;
   r->me2 = me2;
   r->flags = flags;
-  // cost model: the process's operation count per event (helicity sum), the
-  // FP64 path weighted by its measured slowdown; chunks of about kChunkFlop
-  r->flop_per_event = std::max(1.0, P->prog.flops_per_hel * (double)std::max(1, P->prog.n_hel) *
-                                        (prec == MEA_PREC_FP64 ? kFp64Cost : 1.0));
+  r->flop_per_event = mea::request_cost(P, prec);  // chunks of about kChunkFlop
   int64_t cn = (int64_t)(kChunkFlop / r->flop_per_event) / kChunkQuantum * kChunkQuantum;
   cn = std::min(S->chunk, std::max(kChunkQuantum, cn));
   r->chunk = std::min<int64_t>(std::max<int64_t>(n, 1), cn);
