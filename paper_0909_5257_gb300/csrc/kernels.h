@@ -151,6 +151,9 @@ struct AmpConfig {
 // global memory, both of which live in L1.
 int carveout_percent(const DevProgram& p, const AmpConfig& c);
 
+// CTAs of a straight-line kernel that fit an SM.
+int gen_resident(int registers, int threads, size_t smem, size_t smem_sm);
+
 // The straight-line kernels' tile for a call of n_events (dynamic shared memory for a real of that many bytes).
 AmpConfig gen_spread(const DevProgram& p, const AmpConfig& plan, int64_t n_events, size_t real);
 
