@@ -580,9 +580,10 @@ static mea_status create_process(const int* pdg, int n_ext, const mea_options* o
     P->cf_kp = T.kp;
     P->status = const_cast<int*>(dst);
   }
+  const mea::ColourBase base = mea::find_colour_base(G);
   {
     // diagram -> colour-amplitude coefficients for the tensor-core stage
-    P->jmap = mea::build_jamp_map(G);
+    P->jmap = mea::build_jamp_map(G, &base);
     if (P->jmap.ok) {
       const __half* dt = nullptr;
       if ((e = upload(P, P->jmap.tiles, &dt)) != cudaSuccess ||
@@ -604,7 +605,7 @@ static mea_status create_process(const int* pdg, int n_ext, const mea_options* o
   mea::OrdProgram O;
   if (!(G.family == mea::FAM_GLUON && n_ext == 4)) {
     try {
-      O = mea::build_ordered(G);
+      O = mea::build_ordered(G, &base);
     } catch (const mea::LayoutError&) {
       O = mea::OrdProgram();
     }

@@ -5,55 +5,69 @@
 
 namespace mea {
 
+typedef uint32_t u32;
+typedef uint64_t u64;
+static const u64 kPrime = 2147483647ull;  // 2^31 - 1: x mod it is a sum of 31-bit digits
+
+static inline u32 reduce(u64 x) {  // x < 2^63
+  x = (x & kPrime) + (x >> 31);
+  x = (x & kPrime) + (x >> 31);
+  return (u32)(x >= kPrime ? x - kPrime : x);
+}
+static u32 inverse(u32 a) {
+  u64 r = 1, x = a;
+  for (u64 e = kPrime - 2; e; e >>= 1, x = reduce(x * x))
+    if (e & 1) r = reduce(r * x);
+  return (u32)r;
+}
+// x += f y (mod the prime)
+static void add_multiple(std::vector<u32>& x, u32 f, const std::vector<u32>& y, size_t n) {
+  for (size_t j = 0; j < n; ++j) x[j] = reduce(x[j] + (u64)f * y[j]);
+}
+
 // Base of the rows of C (m x kd small integers): the first rows that no
 // earlier ones generate, and the others as sums of them, by elimination
-// modulo a prime on random combinations of the columns (checked exactly below).  Returns false unless the base is rows 0 .. mb - 1
-// and every coefficient is 0, 1 or -1.
-static bool find_base(const std::vector<int>& C, int m, int kd, int& mb, std::vector<std::vector<int>>& coef) {
-  typedef unsigned long long u64;
-  const u64 P = 2147483647ull;
-  auto inv = [&](u64 a) {
-    u64 r = 1, e = P - 2;
-    for (; e; e >>= 1, a = a * a % P)
-      if (e & 1) r = r * a % P;
-    return r;
-  };
-  const int cols = m + 8;
+// modulo a prime on `cols` random combinations of the columns (checked exactly
+// below).  Returns false unless the base is rows 0 .. mb - 1 and every
+// coefficient is 0, 1 or -1.
+static bool find_base(const std::vector<int>& C, int m, int kd, int cols, int& mb, std::vector<std::vector<int>>& coef) {
   u64 seed = 0x9E3779B97F4A7C15ull;
-  std::vector<u64> X((size_t)m * cols, 0), rnd(cols);
-  for (int d = 0; d < kd; ++d) {
-    for (u64& x : rnd) {  // a linear congruential sequence
-      seed = seed * 6364136223846793005ull + 1442695040888963407ull;
-      x = (seed >> 33) % P;
-    }
-    for (int a = 0; a < m; ++a) {
-      const int c = C[(size_t)a * kd + d];
-      if (!c) continue;
-      const u64 cc = (u64)((c + (long long)P) % (long long)P);
-      for (int j = 0; j < cols; ++j) X[(size_t)a * cols + j] = (X[(size_t)a * cols + j] + cc * rnd[j]) % P;
-    }
+  std::vector<u32> rnd((size_t)kd * cols);
+  for (u32& x : rnd) {  // a linear congruential sequence
+    seed = seed * 6364136223846793005ull + 1442695040888963407ull;
+    x = (u32)((seed >> 33) % kPrime);
   }
-  std::vector<std::vector<u64>> B, T;  // reduced rows and what they are of the base rows
+  std::vector<int64_t> sum((size_t)m * cols, 0);  // below kd max|c| 2^31
+  for (int a = 0; a < m; ++a)
+    for (int d = 0; d < kd; ++d) {
+      const int64_t c = C[(size_t)a * kd + d];
+      if (!c) continue;
+      int64_t* s = &sum[(size_t)a * cols];
+      const u32* x = &rnd[(size_t)d * cols];
+      for (int j = 0; j < cols; ++j) s[j] += c * (int64_t)x[j];
+    }
+  std::vector<std::vector<u32>> B, T;  // reduced rows and what they are of the base rows
   std::vector<int> piv;
   mb = 0;
   coef.clear();
   for (int a = 0; a < m; ++a) {
-    std::vector<u64> r(X.begin() + (size_t)a * cols, X.begin() + (size_t)(a + 1) * cols), c(m, 0);
+    std::vector<u32> r(cols), c(m, 0);
+    for (int j = 0; j < cols; ++j) r[j] = (u32)(((sum[(size_t)a * cols + j] % (int64_t)kPrime) + (int64_t)kPrime) % (int64_t)kPrime);
     for (size_t b = 0; b < B.size(); ++b) {
-      const u64 f = r[piv[b]];
+      const u32 f = r[piv[b]];
       if (!f) continue;
-      for (int j = 0; j < cols; ++j) r[j] = (r[j] + (P - f) * B[b][j]) % P;
-      for (int j = 0; j < mb; ++j) c[j] = (c[j] + f * T[b][j]) % P;
+      add_multiple(r, (u32)kPrime - f, B[b], cols);
+      add_multiple(c, f, T[b], mb);
     }
     int q = -1;
     for (int j = 0; j < cols && q < 0; ++j)
       if (r[j]) q = j;
     if (q >= 0) {
       if (a != mb) return false;  // the base is not a prefix
-      const u64 iv = inv(r[q]);
-      for (u64& x : r) x = x * iv % P;
-      std::vector<u64> tb(m, 0);
-      for (int j = 0; j < mb; ++j) tb[j] = (P - c[j]) % P * iv % P;
+      const u32 iv = inverse(r[q]);
+      for (u32& x : r) x = reduce((u64)x * iv);
+      std::vector<u32> tb(m, 0);
+      for (int j = 0; j < mb; ++j) tb[j] = reduce((u64)(c[j] ? (u32)kPrime - c[j] : 0) * iv);
       tb[mb] = iv;
       B.push_back(r);
       T.push_back(tb);
@@ -63,7 +77,7 @@ static bool find_base(const std::vector<int>& C, int m, int kd, int& mb, std::ve
       std::vector<int> k(m, 0);
       for (int j = 0; j < mb; ++j) {
         if (c[j] == 1) k[j] = 1;
-        else if (c[j] == P - 1) k[j] = -1;
+        else if (c[j] == kPrime - 1) k[j] = -1;
         else if (c[j] != 0) return false;
       }
       coef.push_back(k);
@@ -76,6 +90,13 @@ ColourBase find_colour_base(const Program& p) {
   ColourBase B;
   const int m = p.n_jamp;
   B.mb = m;
+  // The strings of one quark line are independent, those of two lines depend on
+  // each other with other coefficients than 1 and -1: nothing to look for.
+  if (p.family != FAM_GLUON) return B;
+  // (n-2)! of the orderings are independent; that many random combinations and a few
+  // more tell the rows apart (a larger rank would fail the exact check)
+  int rank = 1;
+  for (int k = 2; k <= p.n_ext - 2; ++k) rank *= k;
   int kd = 0;
   for (const Op& op : p.ops) kd += is_amp_op(op.type) ? 1 : 0;
   std::vector<int> C((size_t)m * kd, 0);
@@ -91,7 +112,7 @@ ColourBase find_colour_base(const Program& p) {
   }
   int mb = 0;
   std::vector<std::vector<int>> coef;
-  if (!find_base(C, m, kd, mb, coef) || mb >= m) return B;
+  if (!find_base(C, m, kd, std::min(m, rank) + 8, mb, coef) || mb >= m) return B;
   std::vector<uint16_t> index, term;
   for (int a = mb; a < m; ++a) {
     const std::vector<int>& k = coef[a - mb];

@@ -55,7 +55,6 @@
 #include <cstring>
 #include <numeric>
 
-#include "colour_base.h"
 #include "jamp_gemm.h"
 #include "kernels.h"
 #include "tc_common.cuh"
@@ -484,7 +483,7 @@ __global__ void __launch_bounds__(kThreads, 1) jamp_gemm_kernel(JampGemmArgs g) 
 
 }  // namespace
 
-JampMap build_jamp_map(const Program& p) {
+JampMap build_jamp_map(const Program& p, const ColourBase* known) {
   JampMap M;
   M.m = p.n_jamp;
   int kd = 0;
@@ -524,7 +523,7 @@ JampMap build_jamp_map(const Program& p) {
 
   // base columns: one block of them, their terms and a 64-row stage of their
   // integers must fit (kMaxNC columns do)
-  const ColourBase base = find_colour_base(p);
+  const ColourBase base = known ? *known : find_colour_base(p);
   M.mb = M.m;
   if (base.mb < M.m && base.mb <= kMaxNC && base.term.size() <= 4096) {
     M.mb = base.mb;

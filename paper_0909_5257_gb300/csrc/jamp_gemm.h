@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <vector>
 
+#include "colour_base.h"
 #include "generator.h"
 
 namespace mea {
@@ -41,7 +42,8 @@ struct JampMap {
   std::vector<uint16_t> kk_term;
 };
 
-JampMap build_jamp_map(const Program& p);
+// base: find_colour_base(p), found here when null
+JampMap build_jamp_map(const Program& p, const ColourBase* base = nullptr);
 
 // `ops` (all amplitudes of the program, in its order) with every amplitude's row
 // and weight bits in its colour fields (DevProgram::ops_out).

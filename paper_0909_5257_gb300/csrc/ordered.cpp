@@ -1,8 +1,6 @@
 // Ordered-recursion layout of a process (see ordered.h).
 #include "ordered.h"
 
-#include "colour_base.h"
-
 #include <algorithm>
 #include <cstring>
 #include <map>
@@ -208,7 +206,7 @@ uint32_t word_pattern(const Build& B, const Word& w, const std::vector<uint32_t>
 
 }  // namespace
 
-OrdProgram build_ordered(const Program& P) {
+OrdProgram build_ordered(const Program& P, const ColourBase* known) {
   OrdProgram Q;
   Build B(P, Q);
   const int n = P.n_ext;
@@ -220,7 +218,7 @@ OrdProgram build_ordered(const Program& P) {
 
   if (P.family == FAM_GLUON) {
     check(P.root == n - 1, "root leg");
-    const ColourBase base = find_colour_base(P);
+    const ColourBase base = known ? *known : find_colour_base(P);
     const int n_base = base.mb;
     const std::vector<uint16_t>&kk_index = base.index, &kk_term = base.term;
     const int k = n - 2;  // letters of a fused word

@@ -34,6 +34,7 @@
 #include <cstdint>
 #include <vector>
 
+#include "colour_base.h"
 #include "generator.h"
 
 #ifndef MEA_HD
@@ -102,6 +103,7 @@ struct OrdProgram {
 
 // Throws LayoutError when a word needs a momentum the program's event
 // table does not hold or a table does not fit its type.
-OrdProgram build_ordered(const Program& P);
+// base: find_colour_base(P), found here when null
+OrdProgram build_ordered(const Program& P, const ColourBase* base = nullptr);
 
 }  // namespace mea
