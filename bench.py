@@ -73,14 +73,10 @@ FP64_EVENTS = {"gg>ggggg": 2048, "uu~>ggggg": 8192, "uu>uuggg": 16384}
 CPU_SAMPLE = {"gg>ggggg": 16, "uu~>ggggg": 16, "uu>uuggg": 8}
 REF_PER_STEP = {"gg>ggggg": 4, "uu~>ggggg": 4, "uu>uuggg": 2}
 # ncu (dram__bytes_read.sum + dram__bytes_write.sum) per event of the dominant
-# kernel, from the full-size one-pass ncu capture summarised under profiles/,
-# keyed by (subprocess, stage, amplitude kernel 0 per-lane / 1 helicity-shared
-# / 2 split, threads, events per CTA, grid): a launch in another configuration
-# reports null
-TRAFFIC_BYTES_PER_EVENT = {("gg>ggggg", "amplitudes", 0, 128, 1, 1368): (41.71e9 + 35.25e9) / 2731,
-                           ("gg>ggggg", "amplitudes", 0, 224, 2, 760): (42.30e9 + 35.25e9) / 2731,
-                           ("gg>ggggg", "amplitudes", 1, 128, 4, 456): (3.19e9 + 18.99e9) / 2731,
-                           ("gg>ggggg", "amplitudes", 2, 448, 4, 304): (5.52e9 + 19.09e9) / 2731}
+# kernel, from the capture summarised under profiles/, keyed by (subprocess, stage,
+# amplitude kernel as in AMP_KERNEL_NAMES); the kernel writes its diagram amplitudes
+# once, whatever its launch shape
+TRAFFIC_BYTES_PER_EVENT = {("gg>ggggg", "amplitudes", 3): (0.020e9 + 8.813e9) / 2731}
 
 # ---- device-resident workloads (extra keys) ------------------------------------
 WORKLOADS = {
@@ -531,35 +527,14 @@ def _cdiv(a, b):
     return -(-a // b)
 
 
-def _amp_kernel_kind(tune_result):
-    """Which amplitude kernel the tensor-core path of a process runs: the
-    tuner's choice (0 per-lane interpreter, 1 helicity-shared, 2 split, 3
-    phased), else the untuned default, the phased kernel."""
-    return int(tune_result.get("helicity_shared", 0)) if tune_result else 3
-
-
 AMP_KERNEL_NAMES = {0: "per-lane", 1: "helicity-shared", 2: "split", 3: "phased"}
 
 
-def _jamp_executed_flops(info):
-    """Tensor FLOPs the colour-amplitude GEMM executes per (event, helicity)
-    pair: Re and Im rows x 2 FLOP x padded diagrams x padded colour columns
-    x 3 digit planes (tiles of 64 diagrams, column splits of at most 128).
-    Pure-gluon processes contract (n - 2)! of their (n - 1)!/2 colour
-    amplitudes; chunks without a coefficient of a split are not counted out."""
-    m, kd = info["n_colour_amplitudes"], info["n_diagrams"]
-    if info["n_colour"] == 2 * m:
-        m = m * 2 // (info["n_ext"] - 1)
-    nc = min(128, _cdiv(m, 16) * 16)
-    splits = _cdiv(m, nc)
-    nc = min(nc, _cdiv(_cdiv(m, splits), 16) * 16)
-    return 2 * 2 * (_cdiv(kd, 64) * 64) * (splits * nc) * 3
-
-
-def _lanes_share(info):
-    """Share of the helicity combinations that is evaluated: pure-gluon
-    processes evaluate one of every pair of flipped combinations."""
-    return 0.5 if info["n_colour"] == 2 * info["n_colour_amplitudes"] else 1.0
+def _jamp_executed_flops(kernels):
+    """Tensor FLOPs the colour-amplitude GEMM executes per (event, evaluated
+    helicity combination): Re and Im rows x 2 FLOP x 64 diagrams x the columns of
+    a block x 3 digit planes, for every (block, 64 diagrams) tile it contracts."""
+    return 2 * 2 * 64 * kernels["gemm_columns"] * kernels["gemm_chunks"] * 3
 
 
 def _colour_sum_executed_flops(info):
@@ -655,7 +630,7 @@ def run_serve(args):
             "flagged_fraction": float((fl != 0).float().mean()),
             "diagrams": info["n_diagrams"], "colours": info["n_colour"], "helicities": info["n_hel_nonzero"],
             "stage_ms_per_event": {k2: v[0] for k2, v in stage_ms_ev[name].items()},
-            "amplitude_kernel": AMP_KERNEL_NAMES[_amp_kernel_kind(tune.get(name))] +
+            "amplitude_kernel": AMP_KERNEL_NAMES[P.kernels()["amplitude_kernel"]] +
                                 (", forwarding" if (tune.get(name) or {}).get("forwarding") else ""),
         }
         del mom, out, fl, o64
@@ -667,7 +642,8 @@ def run_serve(args):
     dom_nm, dom_stage = max(share, key=share.get)
     tot_share = sum(share.values())
     info = procs[dom_nm].info
-    H = int(info["n_hel_nonzero"] * _lanes_share(info))  # combinations evaluated
+    kern = procs[dom_nm].kernels()
+    H = kern["helicity_lanes"]  # combinations evaluated
     fl_stage = _stage_flops(info, H)
     peaks, peak_src = _peaks()
     bf16_sus = peaks.get("bf16_tflops_sustained", 1700.0)
@@ -676,18 +652,13 @@ def run_serve(args):
     events_per_launch = SUB_EVENTS[dom_nm] / max(stage_ms_ev[dom_nm][dom_stage][1], 1)
     if dom_stage == "amplitudes":
         tc = tune.get(dom_nm) or {}
-        kind = _amp_kernel_kind(tc)
-        # algorithmic FLOPs of the kernel that ran: the phased, the
-        # helicity-shared and the split kernels evaluate (some) wavefunctions
-        # once per helicity pattern of their legs
-        per_event = {1: info["hs_flops_per_event"], 2: info["hsp_flops_per_event"], 3: info["hs_flops_per_event"]}.get(
-            kind, H * fl_stage["amplitudes"])
-        if kind in (1, 2, 3):
-            per_event *= _lanes_share(info)
+        kind = kern["amplitude_kernel"]
+        # FLOPs of the operations that the phased kernel evaluates; the kernels asked
+        # for by helicity_sharing: of the diagrams per combination
+        per_event = kern["phased_flops_per_event"] if kind == 3 else H * fl_stage["amplitudes"]
         flop = events_per_launch * per_event
         achieved = flop / (ms_per_launch * 1e-3) / 1e12
-        tpe = None if tc.get("forwarding") else TRAFFIC_BYTES_PER_EVENT.get(
-            (dom_nm, dom_stage, kind, tc.get("threads"), tc.get("events_per_cta"), tc.get("grid")))
+        tpe = TRAFFIC_BYTES_PER_EVENT.get((dom_nm, dom_stage, kind))
         kname = {1: "amp_hs_kernel<float> (helicity-shared)", 2: "amp_hsp_kernel<float> (split)",
                  3: "amp_phased_kernel (phased)"}.get(
             kind, "amp_kernel<float> amplitude output" + (" with forwarding" if tc.get("forwarding") else ""))
@@ -710,9 +681,10 @@ def run_serve(args):
     tensor = {}
     for nm in names:
         inf = procs[nm].info
-        h = int(inf["n_hel_nonzero"] * _lanes_share(inf))
+        kn = procs[nm].kernels()
+        h = kn["helicity_lanes"]
         f = _stage_flops(inf, h)
-        for stg, exec_flop in (("colour_amplitudes", _jamp_executed_flops(inf)),
+        for stg, exec_flop in (("colour_amplitudes", _jamp_executed_flops(kn)),
                                ("colour_sum", _colour_sum_executed_flops(inf))):
             if stg in stage_ms_ev[nm]:
                 sec = stage_ms_ev[nm][stg][0] * 1e-3  # per event
@@ -938,8 +910,10 @@ def run_device(args):
         name = subs[i][0]
         plain = name in r["tuned"] and not r["tuned"][name]["mixed"].get("vertex_partials", 1)
         return procs[i].info["flops_per_hel_plain" if plain else "flops_per_hel"]
-    cost = [procs[i].info["n_hel_nonzero"] * (body_flops(i) + procs[i].info["colour_flops_per_hel"])
-            for i in range(len(procs))]
+    kern = [P.kernels() for P in procs]
+    cost = [k["helicity_lanes"] * procs[i].info["colour_flops_per_hel"] +
+            (k["phased_flops_per_event"] if k["amplitude_kernel"] == 3 else k["helicity_lanes"] * body_flops(i))
+            for i, k in enumerate(kern)]
     per = r["per_mixed"]
     dom = int(np.argmax([c * statistics.median(per[i]) for i, c in enumerate(cost)]))
     achieved = n * cost[dom] / (statistics.mean(per[dom]) * 1e-3) / 1e12
