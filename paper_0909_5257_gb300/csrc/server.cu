@@ -41,11 +41,11 @@ namespace {
 using Clock = std::chrono::steady_clock;
 
 // Dispatch and chunking constants (see the comment at the top).
-// Target device work of one chunk (request_cost): 1.0 to 1.8 ms of a five-jet process.
-// Measured with the five-jet mix under Poisson arrivals at 0.8 of the capacity, mean /
-// median latency in ms: 1e11 216 / 130, 7e10 216 / 103, 5e10 176 / 60, 4e10 176 / 58;
-// the mix submitted at once takes the same time down to 5e10, 1 % more at 4e10.
-constexpr double kChunkFlop = 5e10;
+// Target device work of one chunk (request_cost): 1.4 to 2.1 ms of a five-jet process.
+// Measured with the five-jet mix, capacity in 1000 events/s, and under Poisson arrivals
+// at 0.8 of it mean / median latency in ms: 1e11 595, 216 / 130; 7e10 591, 218 / 110;
+// 6e10 590, 200 / 88; 5e10 580, 175 / 59 (one median of runs varies by half).
+constexpr double kChunkFlop = 6e10;
 constexpr int64_t kChunkQuantum = 128; // chunk sizes are multiples of this (or the whole request)
 constexpr double kAging = 0.25;        // priority gained per second waited, in seconds of work
 // FP64 path cost relative to the mixed path: whole calls of the five-jet processes
