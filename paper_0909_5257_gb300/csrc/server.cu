@@ -42,9 +42,11 @@ using Clock = std::chrono::steady_clock;
 
 // Dispatch and chunking constants (see the comment at the top).
 // Target device work of one chunk (request_cost): 1.4 to 2.1 ms of a five-jet process.
-// Measured with the five-jet mix, capacity in 1000 events/s, and under Poisson arrivals
-// at 0.8 of it mean / median latency in ms: 1e11 595, 216 / 130; 7e10 591, 218 / 110;
-// 6e10 590, 200 / 88; 5e10 580, 175 / 59 (one median of runs varies by half).
+// Measured with the five-jet mix, capacity in 1000 events/s (60 requests at once; runs of
+// one build differ by 0.6 %), and mean / median latency in ms under Poisson arrivals at
+// 592 k x 0.8 events/s (means of runs of six seeds; medians of runs differ by up to half):
+// three runs of 1e11 595, 210 / 110 and 6e10 591, 197 / 78; two of 7e10 591, 220 / 125,
+// 6e10 590, 200 / 88 and 5e10 580, 173 / 58.
 constexpr double kChunkFlop = 6e10;
 constexpr int64_t kChunkQuantum = 128; // chunk sizes are multiples of this (or the whole request)
 constexpr double kAging = 0.25;        // priority gained per second waited, in seconds of work
