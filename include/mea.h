@@ -430,8 +430,9 @@ mea_status mea_server_destroy(mea_server_t srv);
  *   - A request whose scratch would exceed that size is rejected with
  *     MEA_E_ARG before anything is enqueued (mea_last_error() gives the bytes
  *     needed); for gg -> ggg the flagged-event list limits n_events to about
- *     8.38 million per call, for gg -> gggg the work space to a few hundred
- *     events.
+ *     8.38 million per call, for gg -> gggg the mixed path's work space to a
+ *     few hundred events (its FP64 path runs on as many CTAs as the array
+ *     holds, whatever n_events is).
  *   - The first call on each device (and the first after its CUDA context was
  *     recreated, e.g. by cudaDeviceReset) looks up the array's device address
  *     with that device current; make that first call before any stream

@@ -56,7 +56,8 @@ __host__ __device__ constexpr size_t stage_bytes(int nc) { return (size_t)3 * kP
 // 16 warps instead of 8.  Two where it holds two (nc = 32), which have 16 warps
 // between them already: four leave registers for one CTA only.  Measured,
 // us/event, two -> four: gg>5g 0.613 -> 0.452, uu>uu+3g 0.224 -> 0.179, uu~>5g
-// 0.0957 -> 0.0865, gg>4g 0.020 both; uu~>4g (nc = 32) 0.0146 -> 0.0169.
+// 0.0957 -> 0.0865, gg>4g 0.020 both; uu~>4g (nc = 32) 0.0146 -> 0.0169.  (Making the
+// waits' outcomes uniform over a warp cost 1 to 2 % since.)
 template <int kParts>
 __global__ void __launch_bounds__(kParts * kM, 1) colour_gemm_kernel(ColourGemmArgs g) {
   constexpr int kThreads = kParts * kM;

@@ -151,11 +151,12 @@ Program build_program(const std::vector<int>& pdg, const BuildOptions& opt = Bui
 // Combinations h and n_hel - 1 - h of Program::hel are each other's flips (checked);
 // the lane of both is min(h, n_hel - 1 - h) and evaluates the one whose first leg
 // has helicity -1, so currents holding that leg need half of their variants.
-// Measured on GB300, every combination before, one of each pair now (us per
-// event, whole call): gg>5g 6.14, 3.38; gg>4g 0.301, 0.179; gg>ggg 0.0121,
-// 0.0064; FP64 gg>4g 9.16, 4.59; FP64 gg>gg (2^14 events) 0.0152, 0.0086.  Quark
-// processes keep every combination: their vertex functions order the products
-// of the two chiralities differently, so FP32 results are not the same bits.
+// Measured on GB300 with the kernels of the time, every combination and one of
+// each pair (us per event, whole call): gg>5g 6.14, 3.38; gg>4g 0.301, 0.179;
+// gg>ggg 0.0121, 0.0064; FP64 gg>gg (2^14 events) 0.0152, 0.0086.  (Later steps took
+// gg>5g to 2.67, gg>4g to 0.134, gg>ggg to 0.0040.)  Quark processes keep every
+// combination: their vertex functions order the products of the two chiralities
+// differently, so FP32 results are not the same bits.
 struct HelLanes {
   bool paired = false;
   int n = 0;                 // lanes: n_hel, or n_hel / 2 when paired

@@ -24,12 +24,13 @@
 // words that start with leg 0), the strings of one quark line, or the pairs of
 // strings of two lines, contracted with the integer colour matrix as before.
 //
-// A program is a list of stages with one CTA barrier after each; a stage is a
-// list of words of one form (same number of letters and of helicity bits), an
-// item one word and one helicity pattern.  Patterns are numbered by the
-// letters' bits in word order, the first letter highest.  Currents of as many
-// letters as a colour ordering less one (fused) are not stored: their items
-// close them with the remaining letter at once.
+// A program is a list of stages by level, with one CTA barrier after each level
+// (the stages of a level read nothing that it writes); a stage is a list of words
+// of one form (same number of letters and of helicity bits), an item one word and
+// one helicity pattern.  Patterns are numbered by the letters' bits in word order,
+// the first letter highest.  Currents of as many letters as a colour ordering less
+// one (fused) are not stored: their items close them with the remaining letter at
+// once.
 #pragma once
 #include <cstdint>
 #include <vector>
